@@ -110,7 +110,7 @@ struct JKGraph {
 
 // Exchange-correlation quadrature of a basis (built on first use, kept with the basis): grid points
 // and weights (Becke-partitioned), and every basis function's value and gradient at its molecule's
-// points ([npts_m][n_m] blocks per molecule; gradients as three such blocks).
+// points ([n_m][npts_m] blocks per molecule; gradients as three such blocks).
 struct XcState {
     bool ready = false;
     long long npts = 0, ao = 0, mol_npts_max = 0;
