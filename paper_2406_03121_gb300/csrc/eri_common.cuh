@@ -565,22 +565,28 @@ __device__ __forceinline__ bool warp_uniform_int(int v)
                     }                                                                               \
     }
 
-// Schwarz factors Q_ab = sqrt(max_{m in a, n in b} |(mn|mn)|) for a list of pairs of one class.
+// Schwarz factors Q_ab = sqrt(max_{m in a, n in b} |(mn|mn)|) for a list of pairs of one class, G lanes
+// per pair: the primitive quartets of a diagonal quartet number the square of the pair's primitive
+// pairs (81 in STO-3G, up to 1296 in 6-31G*), so one thread per pair leaves a small molecule waiting for
+// one serial loop.  Lane counts: see schwarz_lanes.  C2H6 / 6-31G's derivative basis, one thread per pair
+// (pp|pp) 13.4 -> 0.43 ms, (ss|ss) 2.1 -> 0.07 ms.
 #define MESS_DEFINE_SCHWARZ_KERNEL(TAG, NA, NB)                                                    \
+    template <int G>                                                                                \
     __global__ void __launch_bounds__(MESS_THREADS)                                                 \
     k_schwarz_##TAG(const int* __restrict__ pairs, int npairs, const PairTable<double> P,           \
                     double* __restrict__ Q)                                                         \
     {                                                                                               \
-        const int t = blockIdx.x * blockDim.x + threadIdx.x;                                        \
-        if (t >= npairs) return;                                                                    \
-        const int p = pairs[t];                                                                     \
+        const int t = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) / G);               \
+        const int g = (int)(threadIdx.x % G);                                                       \
+        if (__all_sync(0xffffffffu, t >= npairs)) return;                                           \
+        const int p = pairs[min(t, npairs - 1)];                                                    \
         double I[(NA) * (NB) * (NA) * (NB)];                                                        \
-        eri_##TAG<double, 0, 1>(P, p, ket_view(P, p, P.rec + p, ket_hdr(P.rec + p)), 0, I);         \
+        eri_##TAG<double, 0, G>(P, p, ket_view(P, p, P.rec + p, ket_hdr(P.rec + p)), g, I, t < npairs); \
         double m = 0.0;                                                                             \
         for (int ia = 0; ia < (NA); ++ia)                                                           \
             for (int ib = 0; ib < (NB); ++ib)                                                       \
                 m = fmax(m, fabs(I[((ia * (NB) + ib) * (NA) + ia) * (NB) + ib]));                   \
-        Q[p] = sqrt(m);                                                                             \
+        if (t < npairs && g == 0) Q[p] = sqrt(m);                                                   \
     }
 
 // ------------------------------------------------------------------------------------------
@@ -694,10 +700,11 @@ template <int TW> __device__ __forceinline__ void team_sync()
 
 // PS (with TW = the block): the block's warps split the quartet's primitive quartets, each warp
 // accumulating into its own copy of the contracted values, summed before the HRR.
+// Evaluates the quartet (bra pair bp, ket view kv) with its TW threads and leaves its integrals in the
+// returned shared-memory array (synchronised).
 template <typename R, int BMODE, int TW, int PS, int L, int NVI, int NH, int NACC, int NVL, int NHL, int NINT,
           int NA, int NB, int NC, int ND>
-__device__ __forceinline__ void jk_team_body(const BinLaunch& b, const PairTable<R>& P, const typename DElem<R>::T* __restrict__ D,
-                                             double* __restrict__ J, double* __restrict__ K, int n,
+__device__ __forceinline__ const R* team_eri(const PairTable<R>& P, int bp, const KetView<R>& kv,
                                              const uint4* __restrict__ vprog, const int* __restrict__ vlev,
                                              const uint2* __restrict__ hprog, const int* __restrict__ hlev,
                                              const int* __restrict__ fslot, const double* __restrict__ fscale,
@@ -708,21 +715,11 @@ __device__ __forceinline__ void jk_team_body(const BinLaunch& b, const PairTable
     static_assert(!PS || TW == 32 * MESS_TEAM_WARPS, "the primitive split spans the block");
     constexpr int TP = PS ? 32 : TW;                // threads of one primitive-loop group
     const int slot = threadIdx.x / TW, lane = threadIdx.x % TW;
-    const long long q = (long long)blockIdx.x * (32 * MESS_TEAM_WARPS / TW) + slot;
-    if (q >= b.total) return;                       // the quartet's threads leave together
     const int pslot = PS ? (int)(threadIdx.x >> 5) : slot, plane = threadIdx.x % TP;
     R* V = sm + (size_t)slot * (NVI + NH);
     R* H = V + NVI;
     R* Vp = sm + (size_t)pslot * (NVI + NH);        // the group's own values and contracted sums
     R* Hp = Vp + NVI;
-    const int i = find_bra(b, q);
-    const int j = __ldg(b.kbeg + i) + (int)(q - __ldg(b.offs + i));
-    const int bp = __ldg(b.bra + i);
-    const KetRec* kr = b.ketrec + j;
-    const int4 kh = ket_hdr(kr);
-    const int kp = ket_pair(kr);
-    if (!P.live(bp) || !P.dens_ok(bp, kp)) return;   // the quartet's threads leave together
-    const KetView<R> kv = ket_view(P, bp, kr, kh);
     for (int k = plane; k < NACC; k += TP) Hp[k] = R(0);
     team_sync<TP>();
     const int b0 = P.pp_off[bp], nbp = P.pp_n[bp];
@@ -803,7 +800,31 @@ __device__ __forceinline__ void jk_team_body(const BinLaunch& b, const PairTable
     }
     for (int k = lane; k < NINT; k += TW) V[k] = gen_scale<R>(fscale, fscale_hi, fscale_lo, k) * H[__ldg(fslot + k)];
     team_sync<TW>();
-    const R* I = V;
+    return V;
+}
+
+template <typename R, int BMODE, int TW, int PS, int L, int NVI, int NH, int NACC, int NVL, int NHL, int NINT,
+          int NA, int NB, int NC, int ND>
+__device__ __forceinline__ void jk_team_body(const BinLaunch& b, const PairTable<R>& P, const typename DElem<R>::T* __restrict__ D,
+                                             double* __restrict__ J, double* __restrict__ K, int n,
+                                             const uint4* __restrict__ vprog, const int* __restrict__ vlev,
+                                             const uint2* __restrict__ hprog, const int* __restrict__ hlev,
+                                             const int* __restrict__ fslot, const double* __restrict__ fscale,
+                                             const float* __restrict__ fscale_hi, const float* __restrict__ fscale_lo,
+                                             R* __restrict__ sm)
+{
+    const int slot = threadIdx.x / TW, lane = threadIdx.x % TW;
+    const long long q = (long long)blockIdx.x * (32 * MESS_TEAM_WARPS / TW) + slot;
+    if (q >= b.total) return;                       // the quartet's threads leave together
+    const int i = find_bra(b, q);
+    const int j = __ldg(b.kbeg + i) + (int)(q - __ldg(b.offs + i));
+    const int bp = __ldg(b.bra + i);
+    const KetRec* kr = b.ketrec + j;
+    const int4 kh = ket_hdr(kr);
+    const int kp = ket_pair(kr);
+    if (!P.live(bp) || !P.dens_ok(bp, kp)) return;   // the quartet's threads leave together
+    const R* I = team_eri<R, BMODE, TW, PS, L, NVI, NH, NACC, NVL, NHL, NINT, NA, NB, NC, ND>(
+        P, bp, ket_view(P, bp, kr, kh), vprog, vlev, hprog, hlev, fslot, fscale, fscale_hi, fscale_lo, sm);
     R s = R(1);
     if (__ldg(P.same + bp)) s *= R(0.5);
     if (kh.w & 1) s *= R(0.5);
@@ -877,6 +898,44 @@ __device__ __forceinline__ void jk_team_body(const BinLaunch& b, const PairTable
                                             reinterpret_cast<R*>(mess_team_smem));                  \
     }
 #define MESS_DEFINE_TEAM_KERNEL(TAG) MESS_DEFINE_TEAM_KERNEL_IMPL(TAG, MESS_TEAM_ARGS_##TAG)
+
+// Schwarz factors of the op-program classes: one block per pair, its warps splitting the primitive
+// quartets of the diagonal quartet.  Latency-bound (81 primitive quartets, one dependency level at a
+// time); C2H6 / 6-31G's derivative basis: (dd|dd) 118.8 -> 1.0 ms, (dp|dp) 106.0 -> 1.4 ms against one
+// thread per pair.
+template <int L, int NVI, int NH, int NACC, int NVL, int NHL, int NINT, int NA, int NB, int NC, int ND>
+__device__ __forceinline__ void schwarz_team_body(const int* __restrict__ pairs, const PairTable<double>& P, double* __restrict__ Q,
+                                                  const uint4* __restrict__ vprog, const int* __restrict__ vlev,
+                                                  const uint2* __restrict__ hprog, const int* __restrict__ hlev,
+                                                  const int* __restrict__ fslot, const double* __restrict__ fscale,
+                                                  const float* __restrict__ fscale_hi, const float* __restrict__ fscale_lo,
+                                                  double* __restrict__ sm)
+{
+    __shared__ double red[MESS_TEAM_WARPS];
+    const int p = pairs[blockIdx.x];
+    const double* I = team_eri<double, 0, 32 * MESS_TEAM_WARPS, 1, L, NVI, NH, NACC, NVL, NHL, NINT, NA, NB, NC, ND>(
+        P, p, ket_view(P, p, P.rec + p, ket_hdr(P.rec + p)), vprog, vlev, hprog, hlev, fslot, fscale, fscale_hi, fscale_lo, sm);
+    double m = 0.0;
+    for (int o = threadIdx.x; o < NA * NB; o += 32 * MESS_TEAM_WARPS) m = fmax(m, fabs(I[o * (NC * ND) + o]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, shfl_xor(m, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < MESS_TEAM_WARPS; ++w) m = fmax(m, red[w]);
+        Q[p] = sqrt(m);
+    }
+}
+
+#define MESS_DEFINE_TEAM_SCHWARZ_KERNEL_IMPL(TAG, ...)                                              \
+    __global__ void __launch_bounds__(32 * MESS_TEAM_WARPS)                                         \
+    k_schwarz_team_##TAG(const int* __restrict__ pairs, const PairTable<double> P, double* __restrict__ Q) \
+    {                                                                                               \
+        extern __shared__ __align__(16) unsigned char mess_team_smem[];                             \
+        schwarz_team_body<__VA_ARGS__>(pairs, P, Q, MESS_TEAM_PROG_##TAG,                           \
+                                       reinterpret_cast<double*>(mess_team_smem));                  \
+    }
+#define MESS_DEFINE_TEAM_SCHWARZ_KERNEL(TAG) MESS_DEFINE_TEAM_SCHWARZ_KERNEL_IMPL(TAG, MESS_TEAM_ARGS_##TAG)
 
 template <typename R, int L, int NVI, int NH, int NACC, int NVL, int NHL, int NINT, int NA, int NB, int NC, int ND>
 constexpr size_t team_smem_bytes()

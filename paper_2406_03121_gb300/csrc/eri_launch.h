@@ -39,6 +39,14 @@ template <> inline const double* dmat<double>(const ClassLaunchArgs& a) { return
 template <> inline const float* dmat<float>(const ClassLaunchArgs& a) { return a.D32; }
 template <> inline const float2* dmat<df32>(const ClassLaunchArgs& a) { return a.Ddf; }
 
+// Lanes per pair of the Schwarz kernels: as few as still give the FP64 pipes four warps per SM (more
+// lanes repeat the per-pair part of the work), 32 where there are too few pairs for that.
+inline int schwarz_lanes(int npairs)
+{
+    const long long fill = 152LL * 4 * 32;
+    return npairs >= fill ? 1 : (8LL * npairs >= fill ? 8 : 32);
+}
+
 typedef cudaError_t (*mess_class_launcher)(const ClassLaunchArgs&);
 extern const mess_class_launcher MESS_CLASS_LAUNCHERS[MESS_NUM_QCLASS];
 

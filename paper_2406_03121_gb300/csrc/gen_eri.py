@@ -889,15 +889,27 @@ def main(outdir):
         if team:
             u.append(f"MESS_DEFINE_TEAM_KERNEL({t})")
         if diag:
-            u.append(f"MESS_DEFINE_SCHWARZ_KERNEL({t}, {na}, {nb})")
+            u.append(f"MESS_DEFINE_SCHWARZ_KERNEL({t}, {na}, {nb})" if info["mode"] == "straight"
+                     else f"MESS_DEFINE_TEAM_SCHWARZ_KERNEL({t})")
         u += ["", f"cudaError_t mess_launch_{t}(const ClassLaunchArgs& a)", "{",
               "    const int T = MESS_THREADS;",
               "    if (a.kind == MESS_KIND_SCHWARZ) {",
               ]
         if diag:
-            u += ["        if (a.npairs <= 0) return cudaSuccess;",
-                  f"        k_schwarz_{t}<<<(a.npairs + T - 1) / T, T, 0, a.stream>>>(a.pairs, a.npairs, *a.P64_ptr, a.out);",
-                  "        return cudaGetLastError();"]
+            u += ["        if (a.npairs <= 0) return cudaSuccess;"]
+            if info["mode"] == "straight":
+                u += ["        const int lanes = schwarz_lanes(a.npairs);",
+                      "        const unsigned nb = (unsigned)(((long long)a.npairs * lanes + T - 1) / T);",
+                      f"        if (lanes == 1) k_schwarz_{t}<1><<<nb, T, 0, a.stream>>>(a.pairs, a.npairs, *a.P64_ptr, a.out);",
+                      f"        else if (lanes == 8) k_schwarz_{t}<8><<<nb, T, 0, a.stream>>>(a.pairs, a.npairs, *a.P64_ptr, a.out);",
+                      f"        else k_schwarz_{t}<32><<<nb, T, 0, a.stream>>>(a.pairs, a.npairs, *a.P64_ptr, a.out);",
+                      "        return cudaGetLastError();"]
+            else:
+                u += [f"        const size_t smem = team_smem_{t}<double>();",
+                      f"        const cudaError_t e = cudaFuncSetAttribute(k_schwarz_team_{t}, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);",
+                      "        if (e != cudaSuccess) return e;",
+                      f"        k_schwarz_team_{t}<<<a.npairs, 32 * MESS_TEAM_WARPS, smem, a.stream>>>(a.pairs, *a.P64_ptr, a.out);",
+                      "        return cudaGetLastError();"]
         else:
             u += ["        return cudaErrorInvalidValue;"]
         u += ["    }",
