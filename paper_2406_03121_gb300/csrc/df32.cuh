@@ -70,6 +70,29 @@ __device__ __forceinline__ df32 df_sqrt(df32 a)
     return df_fast_two_sum(s, __fdividef(r.hi, 2.f * s));
 }
 
+// a + b for |a| >= |b| (8 instructions instead of 11)
+__device__ __forceinline__ df32 df_add_smaller(df32 a, df32 b)
+{
+    const float s = a.hi + b.hi;
+    const float e = b.hi - (s - a.hi);
+    return df_fast_two_sum(s, e + (a.lo + b.lo));
+}
+
+// a^(-1/2): FP32 reciprocal root, one FP32 Newton step, then y (1 + r/2 + 3/8 r^2) with r = 1 - a y^2
+// (|r| < 2e-7) formed to double-float accuracy.  a > 0.
+__device__ __forceinline__ df32 df_rsqrt(df32 a)
+{
+    float y = rsqrtf(a.hi);
+    y = fmaf(0.5f * y, fmaf(-a.hi * y, y, 1.0f), y);
+    const float ph = y * y, pl = fmaf(y, y, -ph);
+    const float mh = a.hi * ph;
+    float ml = fmaf(a.hi, ph, -mh);
+    ml = fmaf(a.hi, pl, ml);
+    ml = fmaf(a.lo, ph, ml);
+    const float r = (1.0f - mh) - ml;
+    return df_fast_two_sum(y, y * (r * fmaf(0.375f, r, 0.5f)));
+}
+
 __device__ __forceinline__ df32 df_shfl_xor(df32 v, int o)
 {
     return df32(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));

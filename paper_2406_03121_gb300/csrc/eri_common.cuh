@@ -97,10 +97,9 @@ template <typename R> struct PairTable {
     const int* __restrict__ mol;             // [npair] molecule of the pair (batched bases)
     const long long* __restrict__ mbase;     // [nmol] offset of the molecule's n x n block (packed matrices)
     const int* __restrict__ mn;              // [nmol] basis functions of the molecule (row stride)
-    const double* __restrict__ boys64;       // Boys grid, FP64
-    const float* __restrict__ boys32;        // Boys grid, FP32
+    const double* __restrict__ boys64;       // FP64 Boys rows per order L (mess_device.h)
     const float4* __restrict__ boys32v;      // FP32 rows per order L: [L][row] {F_L, F_L+1, F_L+2, exp(-T_k)}
-    const float2* __restrict__ boysdf;       // Boys grid, double-float (hi, lo)
+    const float4* __restrict__ boysdf;       // double-float rows per order L
     // per molecule: 0 = left the computation (a converged molecule of a batched SCF): its quartets
     // are skipped by the J/K kernels.  Null: every molecule takes part.
     const unsigned char* __restrict__ active = nullptr;
@@ -211,47 +210,48 @@ __device__ __forceinline__ KetView<df32> ket_view(const PairTable<df32>& P, int 
 __device__ __forceinline__ int ket_pair(const KetRec* r) { return __ldg(&r->pair); }
 
 // ------------------------------------------------------------------------------------------
-// Boys function F_m(T) = int_0^1 t^{2m} exp(-T t^2) dt, m = 0..L.
-// Grid tables tab[k][n] = F_n(k dT) for n = 0..MESS_BOYS_NF-1 and tab[k][MESS_BOYS_NF] = exp(-k dT).
-//   small T: Taylor expansion about the nearest grid point, F_n(T) = sum_j F_{n+j}(T_k) (-x)^j / j!,
-//            x = T - T_k (|x| <= dT/2), for the highest order L, then the stable downward recursion
+// Boys function F_m(T) = int_0^1 t^{2m} exp(-T t^2) dt, m = 0..L, times a factor (the primitive
+// quartet's prefactor).
+//   small T: Taylor expansion about the nearest grid point, F_n(T) = sum_j F_{n+j}(T_k) x^j / j!,
+//            x = T_k - T, for the highest order L, then the stable downward recursion
 //            F_{m-1} = (2 T F_m + exp(-T)) / (2m - 1);
 //   large T: F_0 = (1/2) sqrt(pi/T) (erf(sqrt T) = 1 to working precision there) and the upward
 //            recursion F_{m+1} = ((2m+1) F_m - exp(-T)) / (2T), stable for large T.
-// BMODE 0: everything in FP64.  BMODE 1: FP64 for T < MESS_BOYS_TMAX64 (small-T Taylor + downward
+// The FP64 and double-float forms are bound by instruction count (an FP64 instruction takes 16 cycles of
+// an SM, a double-float operation 7 to 11 instructions), so the grids are fine and their rows hold the
+// Taylor coefficients themselves: 13 FP64 instructions before the recursion, where a step of 0.1 and
+// plain values took 30; 130 FP32 instructions instead of 420 in double-float.
+// BMODE 0: everything in FP64.  BMODE 1: FP64 for T < MESS_BOYS_TMAXDF (small-T Taylor + downward
 // recursion), FP32 asymptote above it.  BMODE 2: everything in FP32.
 // ------------------------------------------------------------------------------------------
-template <int L> __device__ __forceinline__ void boys_small_f64(double T, double* F, const double* __restrict__ c_boys64)
+template <int L> __device__ __forceinline__ void boys_small_f64(double T, double pref, double* F, const double* __restrict__ tab)
 {
-    const int k = __double2int_rn(T * MESS_BOYS_INV_DT);
-    const double x = (double)k * MESS_BOYS_DT - T;      // = -(T - T_k)
-    const double* row = c_boys64 + (size_t)k * MESS_BOYS_NCOL;
-    if (L == 0) {
-        double s = __ldg(row + 7);
-#pragma unroll
-        for (int j = 7; j >= 1; --j) s = __ldg(row + j - 1) + s * x * (1.0 / j);
-        F[0] = s;
-        return;
-    }
-    double s = __ldg(row + L + 7);
-#pragma unroll
-    for (int j = 7; j >= 1; --j) s = __ldg(row + L + j - 1) + s * x * (1.0 / j);
-    F[L] = s;
-    // exp(-T) = exp(-T_k) * exp(x), exp(x) by its Taylor series (|x| <= 0.05)
-    double ex = 1.0 + x * (1.0 + x * (1.0 / 2 + x * (1.0 / 6 + x * (1.0 / 24 + x * (1.0 / 120
-                + x * (1.0 / 720 + x * (1.0 / 5040 + x * (1.0 / 40320))))))));
-    const double e = __ldg(row + MESS_BOYS_NF) * ex;
+    // nearest grid index without conversion instructions (they run on the FP64 pipe): adding 1.5 * 2^52
+    // rounds 32 T to an integer held in the low mantissa bits
+    const double r = fma(T, MESS_BOYS64_INV_DT, 6755399441055744.0);
+    const int k = __double2loint(r);
+    const double x = fma(r - 6755399441055744.0, 1.0 / MESS_BOYS64_INV_DT, -T);
+    const double2* row = reinterpret_cast<const double2*>(tab) + (size_t)(L * MESS_BOYS64_NROW + k) * 4;
+    const double2 a = __ldg(row), b = __ldg(row + 1), c = __ldg(row + 2), d = __ldg(row + 3);
+    const double s = a.x + x * (a.y + x * (b.x + x * (b.y + x * (c.x + x * (c.y + x * d.x)))));
+    F[L] = pref * s;
+    if (L == 0) return;
+    // exp(-T) = exp(-T_k) exp(x) (|x| <= 1/64)
+    const double ex = 1.0 + x * (1.0 + x * (1.0 / 2 + x * (1.0 / 6 + x * (1.0 / 24 + x * (1.0 / 120 + x * (1.0 / 720))))));
+    const double e = pref * d.y * ex;
     const double t2 = 2.0 * T;
 #pragma unroll
-    for (int m = L; m >= 1; --m) F[m - 1] = (t2 * F[m] + e) * (1.0 / (2 * m - 1));
+    for (int m = L; m >= 1; --m) F[m - 1] = m == 1 ? t2 * F[m] + e : (t2 * F[m] + e) * (1.0 / (2 * m - 1));
 }
 
-template <int L> __device__ __forceinline__ void boys_large_f64(double T, double* F)
+// T >= MESS_BOYS_TMAX64: exp(-T) is below 2e-21 there and enters F_8 (4e-11) at 5e-13 of its value, so
+// an FP32 exponential carries it
+template <int L> __device__ __forceinline__ void boys_large_f64(double T, double pref, double* F)
 {
     const double rt = rsqrt(T);
-    F[0] = 0.886226925452758014 * rt;   // sqrt(pi)/2 / sqrt(T)
+    F[0] = 0.886226925452758014 * rt * pref;   // sqrt(pi)/2 / sqrt(T)
     if (L > 0) {
-        const double e = exp(-T);
+        const double e = (double)__expf(-(float)T) * pref;
         const double h = 0.5 * rt * rt;
 #pragma unroll
         for (int m = 0; m < L; ++m) F[m + 1] = ((2 * m + 1) * F[m] - e) * h;
@@ -308,106 +308,95 @@ template <int L> __device__ __forceinline__ void boys_large_f32(float T, float* 
     }
 }
 
-// double-float Boys: the same grid expansion and recursions in df32 arithmetic (grid in hi/lo
-// pairs); above the grid F_0 = sqrt(pi)/2 T^-1/2 and the upward recursion, whose exp(-T) term
-// (below 3e-16 there) is taken in FP32.
+// double-float Boys: the same scheme; terms too small to need it are FP32.  Above the grid F_0 =
+// sqrt(pi)/2 T^-1/2 and the upward recursion, whose exp(-T) term (below 3e-16 there) is FP32.
 __device__ __forceinline__ df32 df_inv_int(int j)   // 1/j as double-float
 {
     const float h = 1.0f / (float)j;
     return df32(h, fmaf(-h, (float)j, 1.0f) / (float)j);
 }
 
-template <int L> __device__ __forceinline__ void boys_small_df(df32 T, df32* F, const float2* __restrict__ tab)
+template <int L> __device__ __forceinline__ void boys_small_df(df32 T, df32 pref, df32* F, const float4* __restrict__ tab)
 {
-    const float r = fmaf(T.hi, (float)MESS_BOYS_INV_DT, 12582912.0f);
+    const float r = fmaf(T.hi, (float)MESS_BOYSDF_INV_DT, 12582912.0f);
     const int k = __float_as_int(r) - 0x4B400000;
-    const df32 dt(0.1f, -1.490116119384765625e-9f);   // 0.1 = hi + lo to 48 bits
-    const df32 x = df32(k) * dt - T;                  // T_k - T
-    const float2* row = tab + (size_t)k * MESS_BOYS_NCOL;
-    const float2 t7 = __ldg(row + L + 7);
-    df32 s(t7.x, t7.y);
-#pragma unroll
-    for (int j = 7; j >= 1; --j) {
-        const float2 tj = __ldg(row + L + j - 1);
-        s = df32(tj.x, tj.y) + s * x * df_inv_int(j);
-    }
-    F[L] = s;
+    // T_k - T.hi is exact (T_k is a short number within 1/128 of T.hi)
+    const float xh = (r - 12582912.0f) * (1.0f / (float)MESS_BOYSDF_INV_DT) - T.hi;
+    const df32 x = df_fast_two_sum(xh, -T.lo);
+    const float4* row = tab + (size_t)(L * MESS_BOYSDF_NROW + k) * 3;
+    const float4 a = __ldg(row), b = __ldg(row + 1), c = __ldg(row + 2);
+    df32 s = df_fast_two_sum(b.z, fmaf(x.hi, fmaf(x.hi, c.y, c.x), b.w));
+    s = df_add_smaller(df32(b.x, b.y), x * s);
+    s = df_add_smaller(df32(a.z, a.w), x * s);
+    s = df_add_smaller(df32(a.x, a.y), x * s);
+    F[L] = pref * s;
     if (L == 0) return;
-    df32 ex = df32(1.0f, 0.f);
+    // exp(x) = 1 + x + x^2/2 + x^3/6 in double-float, x^4/24 + x^5/120 (below 2e-10) in FP32
+    const df32 x2 = x * x, h2 = df32(0.5f * x2.hi, 0.5f * x2.lo);
+    df32 u = df_inv_int(6) * x;
+    u.lo = fmaf(x2.hi, fmaf(x.hi, 1.0f / 120, 1.0f / 24), u.lo);
+    u = df_add_smaller(h2, x2 * df_fast_two_sum(u.hi, u.lo));
+    u = df_add_smaller(x, u);
+    const df32 e = pref * (df32(c.z, c.w) * df_add_smaller(df32(1.0f, 0.f), u));
+    const df32 t2 = df32(2.0f * T.hi, 2.0f * T.lo);
 #pragma unroll
-    for (int j = 9; j >= 1; --j) ex = df32(1.0f, 0.f) + x * df_inv_int(j) * ex;
-    const float2 te = __ldg(row + MESS_BOYS_NF);
-    const df32 e = df32(te.x, te.y) * ex;
-    const df32 t2 = T + T;
-#pragma unroll
-    for (int m = L; m >= 1; --m) F[m - 1] = (t2 * F[m] + e) * df_inv_int(2 * m - 1);
+    for (int m = L; m >= 1; --m) F[m - 1] = m == 1 ? t2 * F[m] + e : (t2 * F[m] + e) * df_inv_int(2 * m - 1);
 }
 
-template <int L> __device__ __forceinline__ void boys_large_df(df32 T, df32* F)
+template <int L> __device__ __forceinline__ void boys_large_df(df32 T, df32 pref, df32* F)
 {
-    const df32 rt = df32(1.0f, 0.f) / df_sqrt(T);
-    F[0] = df32(0.8862269520759583f, -2.6623199644859596e-08f) * rt;   // sqrt(pi)/2 = 0.88622692545275801 as hi + lo
+    const df32 rt = df_rsqrt(T);
+    F[0] = df32(0.8862269520759583f, -2.6623199644859596e-08f) * rt * pref;   // sqrt(pi)/2 = 0.88622692545275801 as hi + lo
     if (L > 0) {
-        const df32 e(__expf(-T.hi), 0.f);
-        const df32 h = df32(0.5f, 0.f) / T;
+        const df32 e = df32(__expf(-T.hi), 0.f) * pref;
+        df32 h = rt * rt;
+        h = df32(0.5f * h.hi, 0.5f * h.lo);
 #pragma unroll
-        for (int m = 0; m < L; ++m) F[m + 1] = (df32(2 * m + 1) * F[m] - e) * h;
+        for (int m = 0; m < L; ++m) F[m + 1] = (df32((float)(2 * m + 1), 0.f) * F[m] - e) * h;
     }
 }
 
-template <typename R> struct PairTable;
+// F_0..F_L times pref
+template <typename R, int L, int BMODE> struct BoysEval;
+template <int L> struct BoysEval<double, L, 0> {
+    static __device__ __forceinline__ void run(double T, double pref, double* F, const PairTable<double>& P)
+    { if (T < MESS_BOYS_TMAX64) boys_small_f64<L>(T, pref, F, P.boys64); else boys_large_f64<L>(T, pref, F); }
+};
+template <int L> struct BoysEval<float, L, 1> {
+    static __device__ __forceinline__ void run(float T, float pref, float* F, const PairTable<float>& P)
+    {
+        if (T < (float)MESS_BOYS_TMAXDF) {
+            double Fd[L + 1];
+            boys_small_f64<L>((double)T, 1.0, Fd, P.boys64);
+#pragma unroll
+            for (int m = 0; m <= L; ++m) F[m] = (float)Fd[m];
+        } else {
+            boys_large_f32<L>(T, F);
+        }
+#pragma unroll
+        for (int m = 0; m <= L; ++m) F[m] *= pref;
+    }
+};
+template <int L> struct BoysEval<float, L, 2> {
+    static __device__ __forceinline__ void run(float T, float pref, float* F, const PairTable<float>& P)
+    {
+        if (T < (float)MESS_BOYS_TMAX32) boys_small_f32<L>(T, F, P.boys32v); else boys_large_f32<L>(T, F);
+#pragma unroll
+        for (int m = 0; m <= L; ++m) F[m] *= pref;
+    }
+};
+template <int L> struct BoysEval<df32, L, 3> {
+    static __device__ __forceinline__ void run(df32 T, df32 pref, df32* F, const PairTable<df32>& P)
+    { if (T < MESS_BOYS_TMAXDF) boys_small_df<L>(T, pref, F, P.boysdf); else boys_large_df<L>(T, pref, F); }
+};
 template <typename R, int L, int BMODE>
-__device__ __forceinline__ void boys_eval(R T, R* F, const PairTable<R>& P);
+__device__ __forceinline__ void boys_eval(R T, R pref, R* F, const PairTable<R>& P) { BoysEval<R, L, BMODE>::run(T, pref, F, P); }
 
-template <> __device__ __forceinline__ void boys_eval<double, 0, 0>(double T, double* F, const PairTable<double>& P)
-{ if (T < MESS_BOYS_TMAX64) boys_small_f64<0>(T, F, P.boys64); else boys_large_f64<0>(T, F); }
-
-#define MESS_BOYS_SPECIALISE(LL)                                                                  \
-    template <> __device__ __forceinline__ void boys_eval<double, LL, 0>(double T, double* F,     \
-                                                                        const PairTable<double>& P) \
-    { if (T < MESS_BOYS_TMAX64) boys_small_f64<LL>(T, F, P.boys64); else boys_large_f64<LL>(T, F); } \
-    template <> __device__ __forceinline__ void boys_eval<float, LL, 1>(float T, float* F,        \
-                                                                       const PairTable<float>& P) \
-    {                                                                                             \
-        if (T < (float)MESS_BOYS_TMAX64) {                                                        \
-            double Fd[LL + 1];                                                                    \
-            boys_small_f64<LL>((double)T, Fd, P.boys64);                                          \
-            _Pragma("unroll") for (int m = 0; m <= LL; ++m) F[m] = (float)Fd[m];                  \
-        } else {                                                                                  \
-            boys_large_f32<LL>(T, F);                                                             \
-        }                                                                                         \
-    }                                                                                             \
-    template <> __device__ __forceinline__ void boys_eval<float, LL, 2>(float T, float* F,        \
-                                                                       const PairTable<float>& P) \
-    { if (T < (float)MESS_BOYS_TMAX32) boys_small_f32<LL>(T, F, P.boys32v); else boys_large_f32<LL>(T, F); } \
-    template <> __device__ __forceinline__ void boys_eval<df32, LL, 3>(df32 T, df32* F,           \
-                                                                      const PairTable<df32>& P)   \
-    { if (T < MESS_BOYS_TMAX64) boys_small_df<LL>(T, F, P.boysdf); else boys_large_df<LL>(T, F); }
-
-MESS_BOYS_SPECIALISE(1)
-MESS_BOYS_SPECIALISE(2)
-MESS_BOYS_SPECIALISE(3)
-MESS_BOYS_SPECIALISE(4)
-MESS_BOYS_SPECIALISE(5)
-MESS_BOYS_SPECIALISE(6)
-MESS_BOYS_SPECIALISE(7)
-MESS_BOYS_SPECIALISE(8)
-
-template <> __device__ __forceinline__ void boys_eval<float, 0, 1>(float T, float* F, const PairTable<float>& P)
-{
-    if (T < (float)MESS_BOYS_TMAX64) { double Fd[1]; boys_small_f64<0>((double)T, Fd, P.boys64); F[0] = (float)Fd[0]; }
-    else boys_large_f32<0>(T, F);
-}
-template <> __device__ __forceinline__ void boys_eval<float, 0, 2>(float T, float* F, const PairTable<float>& P)
-{ if (T < (float)MESS_BOYS_TMAX32) boys_small_f32<0>(T, F, P.boys32v); else boys_large_f32<0>(T, F); }
-template <> __device__ __forceinline__ void boys_eval<df32, 0, 3>(df32 T, df32* F, const PairTable<df32>& P)
-{ if (T < MESS_BOYS_TMAX64) boys_small_df<0>(T, F, P.boysdf); else boys_large_df<0>(T, F); }
-
-// 1/(zeta + eta) and its square root (the prefactor's 1/sqrt(zeta + eta)).  FP32: one reciprocal
-// square root (a few ulp, within the FP32 path's rounding) instead of a division and a square root.
-__device__ __forceinline__ void recip_and_sqrt(double s, double& rz, double& sq) { rz = 1.0 / s; sq = sqrt(rz); }
+// 1/(zeta + eta) and its square root (the prefactor's 1/sqrt(zeta + eta)): one reciprocal square root and
+// its square, instead of a division and a root (FP64: 8 instructions of the FP64 pipe instead of about 20)
+__device__ __forceinline__ void recip_and_sqrt(double s, double& rz, double& sq) { sq = rsqrt(s); rz = sq * sq; }
 __device__ __forceinline__ void recip_and_sqrt(float s, float& rz, float& sq) { sq = rsqrtf(s); rz = sq * sq; }
-__device__ __forceinline__ void recip_and_sqrt(df32 s, df32& rz, df32& sq) { rz = df32(1.0f, 0.f) / s; sq = df_sqrt(rz); }
+__device__ __forceinline__ void recip_and_sqrt(df32 s, df32& rz, df32& sq) { sq = df_rsqrt(s); rz = sq * sq; }
 
 // primitive loops of the straight-line FP32 kernels run two primitive quartets per iteration (more
 // independent loads in flight); FP64 and double-float keep one (register pressure)
@@ -639,9 +628,7 @@ __device__ __forceinline__ void eri_program(const PairTable<R>& P, int bp, const
             const R T = pb.zeta * roz * (PQx * PQx + PQy * PQy + PQz * PQz);
             const R pref = pb.K * pk.K * srz;
             R F[L + 1];
-            boys_eval<R, L, BMODE>(T, F, P);
-#pragma unroll
-            for (int m = 0; m <= L; ++m) F[m] *= pref;
+            boys_eval<R, L, BMODE>(T, pref, F, P);
 #pragma unroll 1
             for (int o = 0; o < NVOPS; ++o) {
                 const uint4 w = __ldg(vprog + o);
@@ -740,9 +727,7 @@ __device__ __forceinline__ const R* team_eri(const PairTable<R>& P, int bp, cons
             const R T = pb.zeta * roz * (PQx * PQx + PQy * PQy + PQz * PQz);
             const R pref = pb.K * pk.K * srz;
             R F[L + 1];
-            boys_eval<R, L, BMODE>(T, F, P);
-#pragma unroll
-            for (int m = 0; m <= L; ++m) F[m] *= pref;
+            boys_eval<R, L, BMODE>(T, pref, F, P);
 #pragma unroll 1
             for (int lv = 0; lv < NVL; ++lv) {
                 const int oend = __ldg(vlev + lv + 1);

@@ -614,9 +614,7 @@ def emit_class_straight(cls):
     body.append("            const R T = pb.zeta * roz * (PQx * PQx + PQy * PQy + PQz * PQz);")
     body.append("            const R pref = pb.K * pk.K * srz;")
     body.append(f"            R F[{L + 1}];")
-    body.append(f"            boys_eval<R, {L}, BMODE>(T, F, P);")
-    body.append("#pragma unroll")
-    body.append(f"            for (int m = 0; m <= {L}; ++m) F[m] *= pref;")
+    body.append(f"            boys_eval<R, {L}, BMODE>(T, pref, F, P);")
     vflops = v.emit(body, "            ")
     for ei, e in enumerate(v.es):
         for fi, f in enumerate(v.fs):

@@ -675,28 +675,8 @@ static mess_status build_pairs(mess_basis* b)
         r.pair = p;
     }
     MESS_CUDA_TRY(b->d_pair_rec.upload(b->pair_rec));
-    std::vector<double> tab;
-    mess_boys_table(tab, MESS_BOYS_NROW, MESS_BOYS_DT);
-    MESS_CUDA_TRY(b->d_boys64.upload(tab));
-    std::vector<float> tab32(tab.begin(), tab.end());
-    MESS_CUDA_TRY(b->d_boys32.upload(tab32));
-    // FP32 rows per order L on the finer grid, one float4 per row: F_L, F_L+1, F_L+2, exp(-T_k)
-    std::vector<double> fine;
-    mess_boys_table(fine, MESS_BOYS32_NROW, MESS_BOYS32_DT);
-    std::vector<float4> tabv((size_t)MESS_BOYS_NL * MESS_BOYS32_NROW);
-    for (int L = 0; L < MESS_BOYS_NL; ++L)
-        for (int k = 0; k < MESS_BOYS32_NROW; ++k) {
-            const double* row = fine.data() + (size_t)k * MESS_BOYS_NCOL;
-            tabv[(size_t)L * MESS_BOYS32_NROW + k] =
-                make_float4((float)row[L], (float)row[L + 1], (float)row[L + 2], (float)row[MESS_BOYS_NF]);
-        }
-    MESS_CUDA_TRY(b->d_boys32v.upload(tabv));
-    std::vector<float2> tabdf(tab.size());
-    for (size_t i = 0; i < tab.size(); ++i) {
-        tabdf[i].x = (float)tab[i];
-        tabdf[i].y = (float)(tab[i] - (double)tabdf[i].x);
-    }
-    MESS_CUDA_TRY(b->d_boysdf.upload(tabdf));
+    MessBoysTables boys;
+    { const mess_status bs = mess_boys_device(&boys); if (bs != MESS_OK) return bs; }
     MESS_CUDA_TRY(b->d_pair_mol.upload(b->pair_mol));
     MESS_CUDA_TRY(b->d_mol_base.upload(b->mol_base));
     MESS_CUDA_TRY(b->d_mol_n.upload(b->mol_nbf));
@@ -718,17 +698,14 @@ static mess_status build_pairs(mess_basis* b)
     b->P64.rec = b->P32.rec = b->Pdf.rec = b->d_pair_rec.p;
     b->P64.mbase = b->P32.mbase = b->d_mol_base.p;
     b->P64.mn = b->P32.mn = b->d_mol_n.p;
-    b->P64.boys64 = b->P32.boys64 = b->d_boys64.p;
-    b->P64.boys32 = b->P32.boys32 = b->d_boys32.p;
-    b->P64.boys32v = b->P32.boys32v = b->d_boys32v.p;
-    b->P64.boysdf = b->P32.boysdf = b->d_boysdf.p;
+    b->P64.boys64 = b->P32.boys64 = b->Pdf.boys64 = boys.b64;
+    b->P64.boys32v = b->P32.boys32v = b->Pdf.boys32v = boys.b32;
+    b->P64.boysdf = b->P32.boysdf = b->Pdf.boysdf = boys.bdf;
     // the double-float table shares every per-pair array with the others
     b->Pdf.pp = b->d_ppdf.p;
     b->Pdf.pp_off = b->P64.pp_off; b->Pdf.pp_n = b->P64.pp_n; b->Pdf.AB = b->P64.AB; b->Pdf.fa = b->P64.fa;
     b->Pdf.fb = b->P64.fb; b->Pdf.same = b->P64.same; b->Pdf.C = b->P64.C; b->Pdf.Cf = b->P64.Cf;
     b->Pdf.ABf = b->P64.ABf; b->Pdf.mol = b->P64.mol; b->Pdf.mbase = b->P64.mbase; b->Pdf.mn = b->P64.mn;
-    b->Pdf.boys64 = b->d_boys64.p; b->Pdf.boys32 = b->d_boys32.p; b->Pdf.boysdf = b->d_boysdf.p;
-    b->Pdf.boys32v = b->d_boys32v.p;
     // shells for the one-electron kernels
     std::vector<int> sl, sK, sf0, spoff;
     std::vector<double> sR, sal, sco;
@@ -811,9 +788,9 @@ static mess_status build_schwarz(mess_basis* b)
 
 void mess_free_basis(mess_basis* b)
 {
-    b->d_pp64.free(); b->d_pp32.free(); b->d_ppdf.free(); b->d_boysdf.free(); b->d_pp_off.free(); b->d_pp_n.free(); b->d_fa.free();
-    b->d_fb.free(); b->d_same.free(); b->d_AB.free(); b->d_Ccen.free(); b->d_ABf.free(); b->d_Cf.free(); b->d_Q.free(); b->d_Qf.free(); b->d_boys64.free();
-    b->d_boys32.free(); b->d_boys32v.free(); b->d_Z.free(); b->d_xyz.free(); b->d_shell_l.free(); b->d_shell_K.free();
+    b->d_pp64.free(); b->d_pp32.free(); b->d_ppdf.free(); b->d_pp_off.free(); b->d_pp_n.free(); b->d_fa.free();
+    b->d_fb.free(); b->d_same.free(); b->d_AB.free(); b->d_Ccen.free(); b->d_ABf.free(); b->d_Cf.free(); b->d_Q.free(); b->d_Qf.free();
+    b->d_Z.free(); b->d_xyz.free(); b->d_shell_l.free(); b->d_shell_K.free();
     b->d_shell_f0.free(); b->d_shell_poff.free(); b->d_shell_R.free(); b->d_shell_alpha.free();
     b->d_shell_coef.free(); b->d_fscale.free(); b->d_pair_a.free(); b->d_pair_b.free();
     b->d_pair_mol.free(); b->d_mol_n.free(); b->d_mol_atom_off.free(); b->d_mol_atom_n.free();

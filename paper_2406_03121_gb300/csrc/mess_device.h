@@ -2,16 +2,25 @@
 #pragma once
 #include <stdint.h>
 
-// Boys-function grid: rows k = 0..MESS_BOYS_NROW-1 at T_k = k * MESS_BOYS_DT; columns n = 0..NF-1
-// hold F_n(T_k) and column NF holds exp(-T_k).
+// Boys-function values reported by mess_boys_grid: rows k = 0..MESS_BOYS_NROW-1 at T_k = k *
+// MESS_BOYS_DT; columns n = 0..NF-1 hold F_n(T_k) and column NF holds exp(-T_k).  The kernels expand
+// around finer grids of the same routine (below), whose steps FP32 and FP64 hold exactly.
 #define MESS_BOYS_DT 0.1
-#define MESS_BOYS_INV_DT 10.0
-#define MESS_BOYS_TMAX64 36.0     // FP64 small-T branch below this (Taylor order 7)
-#define MESS_BOYS_TMAX32 30.0     // FP32 small-T branch below this (Taylor order 4)
+#define MESS_BOYS_TMAX64 48.0     // FP64: Taylor expansion below this
+#define MESS_BOYS_TMAXDF 36.0     // double-float, and the FP64 Boys function of FP32 quartets
+#define MESS_BOYS_TMAX32 30.0     // FP32 (Taylor order 4)
 #define MESS_BOYS_NF 16
 #define MESS_BOYS_NCOL (MESS_BOYS_NF + 1)
 #define MESS_BOYS_NROW 362
 #define MESS_BOYS_NL 9            // orders L = 0..8 of the FP32 Taylor rows (L = la+lb+lc+ld <= 8)
+// FP64 rows: step 1/32 (|T_k - T| <= 1/64, so order 6 leaves 5e-17), per order L and row 64 bytes:
+// F_{L+j}(T_k) / j! for j = 0..6, exp(-T_k).  Double-float rows: step 1/64 (order 5: 3e-16), 48 bytes:
+// the coefficients of j = 0..3 as hi, lo, of j = 4, 5 (whose terms are below 2e-10) as FP32, exp(-T_k)
+// as hi, lo.  With 1/j! in the coefficients a term is one FMA.
+#define MESS_BOYS64_INV_DT 32.0
+#define MESS_BOYS64_NROW 1538
+#define MESS_BOYSDF_INV_DT 64.0
+#define MESS_BOYSDF_NROW 2306
 // FP32 rows: T_k = k * MESS_BOYS32_DT with a step that FP32 holds exactly (1/16: T_k - T is then
 // formed with one rounding; a step of 0.1 or 0.05 rounded to FP32 shifts x by up to 5e-7 at the far
 // end of the grid, a one-signed error of up to 1e-7 in F_L); F_L, F_L+1, F_L+2 and exp(-T_k) in one

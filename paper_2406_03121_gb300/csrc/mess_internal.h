@@ -155,9 +155,6 @@ struct mess_basis {
     DevBuf<double> d_AB, d_Q, d_Ccen;
     DevBuf<float> d_Qf;            // Schwarz factor per pair in FP32 (density screening)
     DevBuf<float> d_ABf, d_Cf;
-    DevBuf<double> d_boys64;
-    DevBuf<float> d_boys32;
-    DevBuf<float4> d_boys32v;
     DevBuf<int> d_Z;
     DevBuf<double> d_xyz;
     DevBuf<int> d_shell_l, d_shell_K, d_shell_f0, d_shell_poff;
@@ -169,7 +166,6 @@ struct mess_basis {
     PairTable<float> P32;
     PairTable<df32> Pdf;
     DevBuf<PrimPairRec<df32>> d_ppdf;
-    DevBuf<float2> d_boysdf;
     BinSet bins;
     // reduced-precision copies of the density of the J/K build in flight (allocated with the bins);
     // a build waits on dconv_free (recorded when the previous build's kernels are done) before
@@ -196,6 +192,9 @@ cudaError_t mess_launch_convert_density(const double* D, float* D32, float2* Ddf
 // Boys tables (boys_table.cu): rows x MESS_BOYS_NCOL
 // F_0..F_{NF-1} and exp(-T) at T_k = k * dt, k < nrow (row-major, MESS_BOYS_NCOL columns)
 void mess_boys_table(std::vector<double>& tab, int nrow, double dt);
+// the kernels' tables on the current device (filled on first use)
+struct MessBoysTables { const double* b64 = nullptr; const float4* b32 = nullptr; const float4* bdf = nullptr; };
+mess_status mess_boys_device(MessBoysTables* out);
 // bins (host.cu)
 mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split);
 // derivative basis (host.cu) of a single-molecule basis whose shells have l < MESS_LMAX: the shells of b

@@ -69,24 +69,6 @@ template <int N, class F> __device__ __forceinline__ void unrolled(F&& f)
     unrolled(f, std::make_integer_sequence<int, N>{});
 }
 
-// F_0..F_L: the kernels' FP64 grid below MESS_BOYS_TMAX64; above it the asymptote and the upward
-// recursion, whose exp(-T) term (below 3e-16 there, F_4 at least 6e-7) needs only FP32 accuracy
-template <int L> __device__ __forceinline__ void boys_1e(double T, double* F, const double* __restrict__ tab)
-{
-    if (T < MESS_BOYS_TMAX64) {
-        boys_small_f64<L>(T, F, tab);
-    } else {
-        const double rt = rsqrt(T);
-        F[0] = 0.886226925452758014 * rt;
-        if (L > 0) {
-            const double e = (double)__expf((float)-T);
-            const double h = 0.5 * rt * rt;
-#pragma unroll
-            for (int m = 0; m < L; ++m) F[m + 1] = ((2 * m + 1) * F[m] - e) * h;
-        }
-    }
-}
-
 // offset of the sums of |e| = L within a lane's sums (which start at |e| = LA)
 template <int LA> __host__ __device__ constexpr int sums_at(int L)
 {
@@ -182,13 +164,10 @@ template <int LA, int LB> __device__ __forceinline__ void one_e_pair(const OneEA
             const double* X = s.xyz + 3 * (at0 + C);
             const double PA[3] = {q.PAx, q.PAy, q.PAz};
             const double PC[3] = {q.PAx + (Rx[0] - X[0]), q.PAy + (Rx[1] - X[1]), q.PAz + (Rx[2] - X[2])};
-            double F[LAB + 1];
-            boys_1e<LAB>(q.zeta * (PC[0] * PC[0] + PC[1] * PC[1] + PC[2] * PC[2]), F, s.P.boys64);
             // 2 pi/p c_a c_b exp(..) = K sqrt(2) pi^(-1/4), K the record's prefactor
             const double pre = -1.0622519320271969 * (double)s.Z[at0 + C] * q.K;
             double t0[1][LAB + 1];
-#pragma unroll
-            for (int m = 0; m <= LAB; ++m) t0[0][m] = pre * F[m];
+            boys_eval<double, LAB, 0>(q.zeta * (PC[0] * PC[0] + PC[1] * PC[1] + PC[2] * PC[2]), pre, t0[0], s.P);
             if (LA == 0) sums[0] += t0[0][0];
             if constexpr (LAB > 0) {
                 double none[1][LAB + 2];
