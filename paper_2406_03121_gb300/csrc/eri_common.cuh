@@ -426,13 +426,31 @@ __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sy
 __device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ df32 shfl_xor(df32 v, int o) { return df_shfl_xor(v, o); }
 
-// sum over aligned groups of G consecutive lanes (G a power of two); every lane of the warp takes part
-template <int G, typename R> __device__ __forceinline__ R group_sum(R v)
-{
+// Sums of acc[0..N) over the G lanes of a group into the group's shared array sh.  Each halving of the
+// group also halves what a lane carries on (it keeps one half and sends the other), so the whole costs
+// about N additions per lane; an all-lanes butterfly of every value takes N log2 G.
+template <int O, int N> struct GroupSums {
+    template <typename R> static __device__ __forceinline__ void run(const R (&acc)[N], int g, int off, int len, R* sh)
+    {
+        constexpr int H = (N + 1) / 2;
+        const bool up = (g & O) != 0;
+        R t[H];
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += shfl_xor(v, o);
-    return v;
-}
+        for (int k = 0; k < H; ++k) {
+            const R lo = acc[k], hi = k + H < N ? acc[k + H < N ? k + H : 0] : R(0);
+            t[k] = (up ? hi : lo) + shfl_xor(up ? lo : hi, O);
+        }
+        GroupSums<O / 2, H>::run(t, g, up ? off + H : off, up ? max(len - H, 0) : min(len, H), sh);
+    }
+};
+template <int N> struct GroupSums<0, N> {
+    template <typename R> static __device__ __forceinline__ void run(const R (&acc)[N], int, int off, int len, R* sh)
+    {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (k < len) sh[off + k] = acc[k];
+    }
+};
 
 template <typename R> __device__ __forceinline__ R warp_sum(R v)
 {
@@ -479,13 +497,81 @@ __device__ __forceinline__ bool warp_uniform_int(int v)
 
 #define MESS_THREADS 128
 
+// Digestion of one quartet by TW threads (this one `lane`): the outputs are dealt out, the integrals are
+// read from shared memory.
+template <typename R, int TW, int NA, int NB, int NC, int ND>
+__device__ __forceinline__ void team_digest(const R* I, const DigestCtx<R>& x, R s, int lane)
+{
+    const typename DElem<R>::T* __restrict__ D = x.D;
+    double* __restrict__ J = x.J;
+    double* __restrict__ K = x.K;
+    const size_t nn = (size_t)x.n;
+    const int fa = x.fa, fb = x.fb, fc = x.fc, fd = x.fd;
+#define MESS_I(a_, b_, c_, d_) I[(((a_) * NB + (b_)) * NC + (c_)) * ND + (d_)]
+    for (int o = lane; o < NA * NB; o += TW) {          // J_ab = sum_cd I D_cd
+        const int a = o / NB, bb = o % NB;
+        R t = R(0);
+        for (int c = 0; c < NC; ++c)
+            for (int d = 0; d < ND; ++d) t += MESS_I(a, bb, c, d) * ldD(D + (fc + c) * nn + fd + d);
+        atomicAdd(J + (fa + a) * nn + fb + bb, to_f64(s * t));
+    }
+    for (int o = lane; o < NC * ND; o += TW) {          // J_cd = sum_ab I D_ab
+        const int c = o / ND, d = o % ND;
+        R t = R(0);
+        for (int a = 0; a < NA; ++a)
+            for (int bb = 0; bb < NB; ++bb) t += MESS_I(a, bb, c, d) * ldD(D + (fa + a) * nn + fb + bb);
+        atomicAdd(J + (fc + c) * nn + fd + d, to_f64(s * t));
+    }
+    for (int o = lane; o < NA * NC; o += TW) {          // K_ac = sum_bd I D_bd
+        const int a = o / NC, c = o % NC;
+        R t = R(0);
+        for (int bb = 0; bb < NB; ++bb)
+            for (int d = 0; d < ND; ++d) t += MESS_I(a, bb, c, d) * ldD(D + (fb + bb) * nn + fd + d);
+        atomicAdd(K + (fa + a) * nn + fc + c, to_f64(s * t));
+    }
+    for (int o = lane; o < NA * ND; o += TW) {          // K_ad = sum_bc I D_bc
+        const int a = o / ND, d = o % ND;
+        R t = R(0);
+        for (int bb = 0; bb < NB; ++bb)
+            for (int c = 0; c < NC; ++c) t += MESS_I(a, bb, c, d) * ldD(D + (fb + bb) * nn + fc + c);
+        atomicAdd(K + (fa + a) * nn + fd + d, to_f64(s * t));
+    }
+    for (int o = lane; o < NB * NC; o += TW) {          // K_bc = sum_ad I D_ad
+        const int bb = o / NC, c = o % NC;
+        R t = R(0);
+        for (int a = 0; a < NA; ++a)
+            for (int d = 0; d < ND; ++d) t += MESS_I(a, bb, c, d) * ldD(D + (fa + a) * nn + fd + d);
+        atomicAdd(K + (fb + bb) * nn + fc + c, to_f64(s * t));
+    }
+    for (int o = lane; o < NB * ND; o += TW) {          // K_bd = sum_ac I D_ac
+        const int bb = o / ND, d = o % ND;
+        R t = R(0);
+        for (int a = 0; a < NA; ++a)
+            for (int c = 0; c < NC; ++c) t += MESS_I(a, bb, c, d) * ldD(D + (fa + a) * nn + fc + c);
+        atomicAdd(K + (fb + bb) * nn + fd + d, to_f64(s * t));
+    }
+#undef MESS_I
+}
+
+// Lanes that share a quartet (G > 1) also share its digestion, through shared memory, where that costs
+// fewer instructions than one lane digesting from registers while the others wait: always in FP64 and
+// double-float (16 cycles or 7 to 11 instructions per operation against about five of addressing and
+// loads), in FP32 from 8 lanes on.
+template <typename R, int G> constexpr bool shared_digest() { return G > 1 && (sizeof(R) == 8 || G >= 8); }
+// shared memory of a group, in elements: its sums, then its integrals; odd, so that groups start in
+// different banks
+constexpr int group_pitch(int nacc, int nint) { return (nacc > nint ? nacc : nint) | 1; }
+
 // JK kernel of one class: G consecutive lanes per shell quartet of the bin (G = 1: one thread).
-#define MESS_DEFINE_CLASS_KERNELS(TAG, NA, NB, NC, ND)                                             \
+#define MESS_DEFINE_CLASS_KERNELS(TAG, NA, NB, NC, ND, NACC)                                       \
     template <typename R, int BMODE, int G>                                                         \
     __global__ void __launch_bounds__(MESS_THREADS)                                                 \
     k_jk_##TAG(const BinLaunch b, const PairTable<R> P, const typename DElem<R>::T* __restrict__ D,            \
                double* __restrict__ J, double* __restrict__ K, int n)                               \
     {                                                                                               \
+        constexpr int NINT_ = (NA) * (NB) * (NC) * (ND), PITCH_ = group_pitch(NACC, NINT_);         \
+        __shared__ __align__(16) unsigned char sh_[G > 1 ? MESS_THREADS / G * PITCH_ * sizeof(R) : 16]; \
+        R* sh = reinterpret_cast<R*>(sh_) + (G > 1 ? (int)threadIdx.x / G * PITCH_ : 0);            \
         const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;                     \
         const long long q0 = t0 / G;                                                                \
         const int g = (int)(t0 % G);                                                                \
@@ -501,8 +587,8 @@ __device__ __forceinline__ bool warp_uniform_int(int v)
         /* quartet to do leaves (lanes of a group share the quartet, so groups leave together)  */ \
         const bool live = valid && P.live(bp) && P.dens_ok(bp, kp);                                 \
         if (__all_sync(0xffffffffu, !live)) return;                                                 \
-        R I[(NA) * (NB) * (NC) * (ND)];                                                             \
-        eri_##TAG<R, BMODE, G>(P, bp, ket_view(P, bp, kr, kh), g, I, live);                        \
+        R I[NINT_];                                                                                 \
+        eri_##TAG<R, BMODE, G>(P, bp, ket_view(P, bp, kr, kh), g, I, live, sh);                    \
         DigestCtx<R> c;                                                                              \
         {                                                                                           \
             const int m_ = __ldg(P.mol + bp);                                                       \
@@ -519,6 +605,11 @@ __device__ __forceinline__ bool warp_uniform_int(int v)
         if (G == 1) {                                                                               \
             c.warp_reduce_ab = warp_uniform_int(bp);                                                \
             digest_##TAG<R>(I, c, s);                                                               \
+        } else if constexpr (shared_digest<R, G>()) {                                               \
+            _Pragma("unroll") for (int k = 0; k < NINT_; ++k)                                       \
+                if (k % G == g) sh[k] = I[k];                                                       \
+            __syncwarp();                                                                           \
+            if (live) team_digest<R, G, NA, NB, NC, ND>(sh, c, s, g);                               \
         } else if (g == 0) {                                                                        \
             c.warp_reduce_ab = false;                                                               \
             digest_##TAG<R>(I, c, s);                                                               \
@@ -559,18 +650,21 @@ __device__ __forceinline__ bool warp_uniform_int(int v)
 // pairs (81 in STO-3G, up to 1296 in 6-31G*), so one thread per pair leaves a small molecule waiting for
 // one serial loop.  Lane counts: see schwarz_lanes.  C2H6 / 6-31G's derivative basis, one thread per pair
 // (pp|pp) 13.4 -> 0.43 ms, (ss|ss) 2.1 -> 0.07 ms.
-#define MESS_DEFINE_SCHWARZ_KERNEL(TAG, NA, NB)                                                    \
+#define MESS_DEFINE_SCHWARZ_KERNEL(TAG, NA, NB, NACC)                                              \
     template <int G>                                                                                \
     __global__ void __launch_bounds__(MESS_THREADS)                                                 \
     k_schwarz_##TAG(const int* __restrict__ pairs, int npairs, const PairTable<double> P,           \
                     double* __restrict__ Q)                                                         \
     {                                                                                               \
+        constexpr int PITCH_ = group_pitch(NACC, 0);                                                \
+        __shared__ double sh[G > 1 ? MESS_THREADS / G * PITCH_ : 1];                                \
         const int t = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) / G);               \
         const int g = (int)(threadIdx.x % G);                                                       \
         if (__all_sync(0xffffffffu, t >= npairs)) return;                                           \
         const int p = pairs[min(t, npairs - 1)];                                                    \
         double I[(NA) * (NB) * (NA) * (NB)];                                                        \
-        eri_##TAG<double, 0, G>(P, p, ket_view(P, p, P.rec + p, ket_hdr(P.rec + p)), g, I, t < npairs); \
+        eri_##TAG<double, 0, G>(P, p, ket_view(P, p, P.rec + p, ket_hdr(P.rec + p)), g, I, t < npairs, \
+                               sh + (G > 1 ? (int)threadIdx.x / G * PITCH_ : 0));                   \
         double m = 0.0;                                                                             \
         for (int ia = 0; ia < (NA); ++ia)                                                           \
             for (int ib = 0; ib < (NB); ++ib)                                                       \
@@ -814,58 +908,12 @@ __device__ __forceinline__ void jk_team_body(const BinLaunch& b, const PairTable
     if (__ldg(P.same + bp)) s *= R(0.5);
     if (kh.w & 1) s *= R(0.5);
     if (bp == kp) s *= R(0.5);
-    const int fa = __ldg(P.fa + bp), fb = __ldg(P.fb + bp), fc = kh.z & 0xffff, fd = kh.z >> 16;
     const int mol_ = __ldg(P.mol + bp);
     const long long off_ = __ldg(P.mbase + mol_);
-    D += off_;
-    J += off_;
-    K += off_;
-    const size_t nn = (size_t)__ldg(P.mn + mol_);
     (void)n;
-#define MESS_I(a_, b_, c_, d_) I[(((a_) * NB + (b_)) * NC + (c_)) * ND + (d_)]
-    for (int o = lane; o < NA * NB; o += TW) {          // J_ab = sum_cd I D_cd
-        const int a = o / NB, bb = o % NB;
-        R t = R(0);
-        for (int c = 0; c < NC; ++c)
-            for (int d = 0; d < ND; ++d) t += MESS_I(a, bb, c, d) * ldD(D + (fc + c) * nn + fd + d);
-        atomicAdd(J + (fa + a) * nn + fb + bb, to_f64(s * t));
-    }
-    for (int o = lane; o < NC * ND; o += TW) {          // J_cd = sum_ab I D_ab
-        const int c = o / ND, d = o % ND;
-        R t = R(0);
-        for (int a = 0; a < NA; ++a)
-            for (int bb = 0; bb < NB; ++bb) t += MESS_I(a, bb, c, d) * ldD(D + (fa + a) * nn + fb + bb);
-        atomicAdd(J + (fc + c) * nn + fd + d, to_f64(s * t));
-    }
-    for (int o = lane; o < NA * NC; o += TW) {          // K_ac = sum_bd I D_bd
-        const int a = o / NC, c = o % NC;
-        R t = R(0);
-        for (int bb = 0; bb < NB; ++bb)
-            for (int d = 0; d < ND; ++d) t += MESS_I(a, bb, c, d) * ldD(D + (fb + bb) * nn + fd + d);
-        atomicAdd(K + (fa + a) * nn + fc + c, to_f64(s * t));
-    }
-    for (int o = lane; o < NA * ND; o += TW) {          // K_ad = sum_bc I D_bc
-        const int a = o / ND, d = o % ND;
-        R t = R(0);
-        for (int bb = 0; bb < NB; ++bb)
-            for (int c = 0; c < NC; ++c) t += MESS_I(a, bb, c, d) * ldD(D + (fb + bb) * nn + fc + c);
-        atomicAdd(K + (fa + a) * nn + fd + d, to_f64(s * t));
-    }
-    for (int o = lane; o < NB * NC; o += TW) {          // K_bc = sum_ad I D_ad
-        const int bb = o / NC, c = o % NC;
-        R t = R(0);
-        for (int a = 0; a < NA; ++a)
-            for (int d = 0; d < ND; ++d) t += MESS_I(a, bb, c, d) * ldD(D + (fa + a) * nn + fd + d);
-        atomicAdd(K + (fb + bb) * nn + fc + c, to_f64(s * t));
-    }
-    for (int o = lane; o < NB * ND; o += TW) {          // K_bd = sum_ac I D_ac
-        const int bb = o / ND, d = o % ND;
-        R t = R(0);
-        for (int a = 0; a < NA; ++a)
-            for (int c = 0; c < NC; ++c) t += MESS_I(a, bb, c, d) * ldD(D + (fa + a) * nn + fc + c);
-        atomicAdd(K + (fb + bb) * nn + fd + d, to_f64(s * t));
-    }
-#undef MESS_I
+    const DigestCtx<R> c{D + off_, J + off_, K + off_, __ldg(P.mn + mol_), __ldg(P.fa + bp), __ldg(P.fb + bp),
+                         kh.z & 0xffff, kh.z >> 16, false};
+    team_digest<R, TW, NA, NB, NC, ND>(I, c, s, lane);
 }
 
 #define MESS_DEFINE_TEAM_KERNEL_IMPL(TAG, ...)                                                      \

@@ -39,6 +39,11 @@ template <> inline const double* dmat<double>(const ClassLaunchArgs& a) { return
 template <> inline const float* dmat<float>(const ClassLaunchArgs& a) { return a.D32; }
 template <> inline const float2* dmat<df32>(const ClassLaunchArgs& a) { return a.Ddf; }
 
+// Threads per block of the straight-line J/K kernels: one warp while the warps are fewer than eight per
+// SM, so that they spread over the SMs (the FP64 pipe of an SM serves one warp instruction in 16 cycles
+// and is full with one block of four warps), else four warps (MESS_THREADS).
+inline int jk_block_threads(long long threads) { return threads < 152LL * 8 * 32 ? 32 : 128; }
+
 // Lanes per pair of the Schwarz kernels: as few as still give the FP64 pipes four warps per SM (more
 // lanes repeat the per-pair part of the work), 32 where there are too few pairs for that.
 inline int schwarz_lanes(int npairs)

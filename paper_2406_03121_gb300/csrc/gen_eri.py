@@ -588,7 +588,7 @@ def emit_class_straight(cls):
     lines = []
     lines.append(f"// ---- class ({la}{lb}|{lc}{ld}): {len(v.order)} VRR entries, {nacc} contracted, {nint} integrals")
     lines.append(f"template <typename R, int BMODE, int G>")
-    lines.append(f"__device__ __forceinline__ void eri_{t}(const PairTable<R>& P, int bp, const KetView<R>& kv, int g, R* I, bool live = true)")
+    lines.append(f"__device__ __forceinline__ void eri_{t}(const PairTable<R>& P, int bp, const KetView<R>& kv, int g, R* I, bool live = true, R* sh = nullptr)")
     lines.append("{")
     lines.append(f"    R acc[{nacc}];")
     lines.append(f"#pragma unroll")
@@ -646,8 +646,11 @@ def emit_class_straight(cls):
     lines.append("        ik += G;")
     lines.append("        while (ik >= k1 && ib < b1) { ik -= nk; ++ib; }")
     lines.append("    }")
+    lines.append(f"    GroupSums<G / 2, {nacc}>::run(acc, g, 0, {nacc}, sh);")
+    lines.append("    __syncwarp();")
     lines.append("#pragma unroll")
-    lines.append(f"    for (int k = 0; k < {nacc}; ++k) acc[k] = group_sum<G>(acc[k]);")
+    lines.append(f"    for (int k = 0; k < {nacc}; ++k) acc[k] = sh[k];")
+    lines.append("    __syncwarp();")
     lines.append("    }")
     lines.append("    const R ABx = pair_ab(P, bp, 0), ABy = pair_ab(P, bp, 1), ABz = pair_ab(P, bp, 2);")
     lines.append("    const R CDx = kv.CD[0], CDy = kv.CD[1], CDz = kv.CD[2];")
@@ -693,15 +696,15 @@ def emit_class(cls):
                    f"slots, {len(pr['hrr'])} HRR ops on {pr['nh']} slots"]
         L += emit_program_tables(t, pr)
         L.append("template <typename R, int BMODE, int G>")
-        L.append(f"__device__ __forceinline__ void eri_{t}(const PairTable<R>& P, int bp, const KetView<R>& kv, int g, R* I, bool live = true)")
+        L.append(f"__device__ __forceinline__ void eri_{t}(const PairTable<R>& P, int bp, const KetView<R>& kv, int g, R* I, bool live = true, R* sh = nullptr)")
         L.append("{")
         L.append("    if constexpr (std::is_same<R, df32>::value && G == 1) {")
-        L.append("        (void)g;")
+        L.append("        (void)g; (void)sh;")
         L.append(f"        eri_program<R, BMODE, {pr['L']}, {pr['nv']}, {pr['nh']}, {pr['nacc']}, {len(pr['vrr'])}, "
                  f"{len(pr['hrr'])}, {len(pr['fin'])}>(P, bp, kv, vprog_{t}, hprog_{t}, fslot_{t}, fscale_{t}, "
                  f"fscaleh_{t}, fscalel_{t}, I, live);")
         L.append("    } else {")
-        L.append(f"        eri_{t}_sl<R, BMODE, G>(P, bp, kv, g, I, live);")
+        L.append(f"        eri_{t}_sl<R, BMODE, G>(P, bp, kv, g, I, live, sh);")
         L.append("    }")
         L.append("}")
         return "\n".join(L) + "\n", info
@@ -713,10 +716,10 @@ def emit_class(cls):
              f"{len(pr['hrr'])} HRR ops on {pr['nh']} slots")
     L += emit_program_tables(t, pr)
     L.append("template <typename R, int BMODE, int G>")
-    L.append(f"__device__ __forceinline__ void eri_{t}(const PairTable<R>& P, int bp, const KetView<R>& kv, int g, R* I, bool live = true)")
+    L.append(f"__device__ __forceinline__ void eri_{t}(const PairTable<R>& P, int bp, const KetView<R>& kv, int g, R* I, bool live = true, R* sh = nullptr)")
     L.append("{")
     L.append("    static_assert(G == 1, \"op-program classes run one thread per quartet\");")
-    L.append("    (void)g;")
+    L.append("    (void)g; (void)sh;")
     L.append(f"    eri_program<R, BMODE, {pr['L']}, {pr['nv']}, {pr['nh']}, {pr['nacc']}, {len(pr['vrr'])}, "
              f"{len(pr['hrr'])}, {len(pr['fin'])}>(P, bp, kv, vprog_{t}, hprog_{t}, fslot_{t}, fscale_{t}, "
              f"fscaleh_{t}, fscalel_{t}, I, live);")
@@ -882,12 +885,12 @@ def main(outdir):
         na, nb, nc, nd = ncart(la), ncart(lb), ncart(lc), ncart(ld)
         diag = (la, lb) == (lc, ld)
         u = ["// Generated by gen_eri.py: do not edit.", f'#include "eri_class_{t}.cuh"', '#include "eri_launch.h"', "",
-             f"MESS_DEFINE_CLASS_KERNELS({t}, {na}, {nb}, {nc}, {nd})"]
+             f"MESS_DEFINE_CLASS_KERNELS({t}, {na}, {nb}, {nc}, {nd}, {info['nacc']})"]
         team = team_capable(info) or info["mode"] == "program"
         if team:
             u.append(f"MESS_DEFINE_TEAM_KERNEL({t})")
         if diag:
-            u.append(f"MESS_DEFINE_SCHWARZ_KERNEL({t}, {na}, {nb})" if info["mode"] == "straight"
+            u.append(f"MESS_DEFINE_SCHWARZ_KERNEL({t}, {na}, {nb}, {info['nacc']})" if info["mode"] == "straight"
                      else f"MESS_DEFINE_TEAM_SCHWARZ_KERNEL({t})")
         u += ["", f"cudaError_t mess_launch_{t}(const ClassLaunchArgs& a)", "{",
               "    const int T = MESS_THREADS;",
@@ -912,11 +915,12 @@ def main(outdir):
             u += ["        return cudaErrorInvalidValue;"]
         u += ["    }",
               "    if (a.bin.total <= 0) return cudaSuccess;",
-              "    const long long nblk = (a.bin.total + T - 1) / T;",
+              "    const int T1 = a.kind == MESS_KIND_JK ? jk_block_threads(a.bin.total) : T;",
+              "    const long long nblk = (a.bin.total + T1 - 1) / T1;",
               "    if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;",
               "    const dim3 g((unsigned)nblk);",
               "    if (a.kind == MESS_KIND_STORE) {",
-              f"        k_store_{t}<<<g, T, 0, a.stream>>>(a.bin, *a.P64_ptr, a.out, a.n);",
+              f"        k_store_{t}<<<g, T1, 0, a.stream>>>(a.bin, *a.P64_ptr, a.out, a.n);",
               "    } else {",
               ] + ([
               "      if (a.team) {",
@@ -959,27 +963,28 @@ def main(outdir):
               ] if (team_capable(info) or info["mode"] == "program") else []) + ([
               ] + sum([[
               f"        if (a.G == {GG}) {{",
-              f"            const long long nbg = (a.bin.total * {GG} + T - 1) / T;",
+              f"            const int TG = jk_block_threads(a.bin.total * {GG});",
+              f"            const long long nbg = (a.bin.total * {GG} + TG - 1) / TG;",
               "            if (nbg > 0x7fffffffLL) return cudaErrorInvalidConfiguration;",
               "            const dim3 gg((unsigned)nbg);",
               "            if (a.mode == MESS_MODE_FP64)",
-              f"                k_jk_{t}<double, 0, {GG}><<<gg, T, 0, a.stream>>>(a.bin, *a.P64_ptr, dmat<double>(a), a.J, a.K, a.n);",
+              f"                k_jk_{t}<double, 0, {GG}><<<gg, TG, 0, a.stream>>>(a.bin, *a.P64_ptr, dmat<double>(a), a.J, a.K, a.n);",
               "            else if (a.mode == MESS_MODE_MIXED)",
-              f"                k_jk_{t}<float, 1, {GG}><<<gg, T, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
+              f"                k_jk_{t}<float, 1, {GG}><<<gg, TG, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
               "            else if (a.mode == MESS_MODE_DF32)",
-              f"                k_jk_{t}<df32, 3, {GG}><<<gg, T, 0, a.stream>>>(a.bin, *a.Pdf_ptr, dmat<df32>(a), a.J, a.K, a.n);",
+              f"                k_jk_{t}<df32, 3, {GG}><<<gg, TG, 0, a.stream>>>(a.bin, *a.Pdf_ptr, dmat<df32>(a), a.J, a.K, a.n);",
               "            else",
-              f"                k_jk_{t}<float, 2, {GG}><<<gg, T, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
+              f"                k_jk_{t}<float, 2, {GG}><<<gg, TG, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
               "            return cudaGetLastError();",
               "        }"] for GG in (4, 8, 32)], []) if info["mode"] == "straight" else []) + [
               "        if (a.mode == MESS_MODE_FP64)",
-              f"            k_jk_{t}<double, 0, 1><<<g, T, 0, a.stream>>>(a.bin, *a.P64_ptr, dmat<double>(a), a.J, a.K, a.n);",
+              f"            k_jk_{t}<double, 0, 1><<<g, T1, 0, a.stream>>>(a.bin, *a.P64_ptr, dmat<double>(a), a.J, a.K, a.n);",
               "        else if (a.mode == MESS_MODE_MIXED)",
-              f"            k_jk_{t}<float, 1, 1><<<g, T, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
+              f"            k_jk_{t}<float, 1, 1><<<g, T1, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
               "        else if (a.mode == MESS_MODE_DF32)",
-              f"            k_jk_{t}<df32, 3, 1><<<g, T, 0, a.stream>>>(a.bin, *a.Pdf_ptr, dmat<df32>(a), a.J, a.K, a.n);",
+              f"            k_jk_{t}<df32, 3, 1><<<g, T1, 0, a.stream>>>(a.bin, *a.Pdf_ptr, dmat<df32>(a), a.J, a.K, a.n);",
               "        else",
-              f"            k_jk_{t}<float, 2, 1><<<g, T, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
+              f"            k_jk_{t}<float, 2, 1><<<g, T1, 0, a.stream>>>(a.bin, *a.P32_ptr, dmat<float>(a), a.J, a.K, a.n);",
               "    }",
               "    return cudaGetLastError();",
               "}"]
