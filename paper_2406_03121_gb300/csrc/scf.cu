@@ -332,35 +332,66 @@ __device__ __forceinline__ void jac_set(double& x, double v) { x = v; }
 __device__ __forceinline__ void jac_set(df32& x, double v) { x = df32(v); }
 __device__ __forceinline__ double jac_get(double x) { return x; }
 __device__ __forceinline__ double jac_get(df32 x) { return f2d_alu(x.hi) + f2d_alu(x.lo); }
-__device__ __forceinline__ double jac_lead(double x) { return x; }            // for tests and sums
-__device__ __forceinline__ double jac_lead(df32 x) { return f2d_alu(x.hi); }
-__device__ __forceinline__ bool jac_iszero(double x) { return x == 0.0; }
-__device__ __forceinline__ bool jac_iszero(df32 x) { return x.hi == 0.f; }
-__device__ __forceinline__ double jac_sqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ df32 jac_sqrt(df32 x) { return df_sqrt(x); }
-__device__ __forceinline__ double jac_abs(double x) { return fabs(x); }
-__device__ __forceinline__ df32 jac_abs(df32 x) { return x.hi < 0.f ? -x : x; }
-template <typename T> __device__ __forceinline__ T jac_one();
-template <> __device__ __forceinline__ double jac_one<double>() { return 1.0; }
-template <> __device__ __forceinline__ df32 jac_one<df32>() { return df32(1.0f, 0.f); }
-template <typename T> __device__ __forceinline__ T jac_zero();
-template <> __device__ __forceinline__ double jac_zero<double>() { return 0.0; }
-template <> __device__ __forceinline__ df32 jac_zero<df32>() { return df32(0.f, 0.f); }
+__device__ __forceinline__ float jac_f32(double x) { return (float)x; }
+__device__ __forceinline__ float jac_f32(df32 x) { return x.hi; }
+template <typename T> __device__ __forceinline__ T jac_const(float v);
+template <> __device__ __forceinline__ double jac_const<double>(float v) { return v; }
+template <> __device__ __forceinline__ df32 jac_const<df32>(float v) { return df32(v, 0.f); }
+// sums of squares for the convergence test: FP64, or FP32 where the threshold is only 1e-25 of the whole
+template <typename T> struct JacSum { typedef double type; };
+template <> struct JacSum<df32> { typedef float type; };
+__device__ __forceinline__ double jac_sq(double x) { return x * x; }
+__device__ __forceinline__ float jac_sq(df32 x) { return x.hi * x.hi; }
+// cosine of the rotation whose tangent is t: (1 + t^2)^(-1/2) to the element type's accuracy
+__device__ __forceinline__ double jac_cos(double, float t) { return rsqrt(fma((double)t, (double)t, 1.0)); }
+__device__ __forceinline__ df32 jac_cos(df32, float t)
+{
+    const float q = t * t;
+    return df_rsqrt(df_add_smaller(df32(1.0f, 0.f), df32(q, fmaf(t, t, -q))));   // |t| <= 1
+}
+__device__ __forceinline__ double jac_scale(double c, float t) { return c * (double)t; }
+__device__ __forceinline__ df32 jac_scale(df32 c, float t)
+{
+    const float p = c.hi * t;
+    return df_fast_two_sum(p, fmaf(c.lo, t, fmaf(c.hi, t, -p)));
+}
+// c x + s y
+__device__ __forceinline__ double jac_comb(double c, double x, double s, double y) { return fma(c, x, s * y); }
+__device__ __forceinline__ df32 jac_comb(df32 c, df32 x, df32 s, df32 y)
+{
+    const float p = c.hi * x.hi, q = s.hi * y.hi;
+    float e = fmaf(c.hi, x.hi, -p) + fmaf(s.hi, y.hi, -q);
+    e = fmaf(c.hi, x.lo, e);
+    e = fmaf(c.lo, x.hi, e);
+    e = fmaf(s.hi, y.lo, e);
+    e = fmaf(s.lo, y.hi, e);
+    const df32 r = df_two_sum(p, q);
+    return df_fast_two_sum(r.hi, r.lo + e);
+}
 // a rotation is skipped when |a_pq| <= JacEps::skip sqrt(|a_pp a_qq|); the sweeps stop when the
 // off-diagonal Frobenius norm squared is below JacEps::off of the whole (relative round-off level)
 template <typename T> struct JacEps;
-template <> struct JacEps<double> { static constexpr double skip = 1e-15, off = 1e-28; };
-template <> struct JacEps<df32> { static constexpr double skip = 1e-13, off = 1e-25; };
+template <> struct JacEps<double> { static constexpr float skip = 1e-15f; static constexpr double off = 1e-28; };
+template <> struct JacEps<df32> { static constexpr float skip = 1e-13f; static constexpr double off = 1e-25; };
+
+constexpr int kJacMaxHalf = 128;   // pairs of a round (n <= 256)
 
 // Cyclic Jacobi eigensolver of the symmetric n x n block of each molecule, one thread block per
 // molecule, rotations in parallel over disjoint index pairs (round-robin "circle" schedule).  The
 // rotation of (p, q) uses tau = (a_qq - a_pp)/(2 a_pq), t = sign(tau)/(|tau| + sqrt(1 + tau^2)),
 // c = 1/sqrt(1 + t^2), s = t c, and A <- J^T A J, V <- V J.  Eigenvalues ascending in eps, the
-// matching eigenvectors as the columns of Vout.  The matrix (element type T, 8 bytes) lives in
-// shared memory when it fits, otherwise in the global workspace Wk.  The eigenvectors accumulate
-// transposed in the global workspace Vt (row k = eigenvector k), so that the update of V's columns
-// p, q runs along contiguous rows.  Each warp takes whole rows (lanes along the row): no index
-// division anywhere in the sweeps.
+// matching eigenvectors as the columns of Vout.
+// A round is bound by its serial chain (rotation angles, barrier, update, barrier) for small matrices
+// and by the instructions of the update for large ones (FP64: the FP64 pipe), so:
+//   - t is taken in FP32 (a rotation by a slightly wrong angle is still a rotation: it leaves 1e-7 of a_pq
+//     for the next sweep); c and s have c^2 + s^2 = 1 to the accuracy of T;
+//   - both sides of the update act on the 2 x 2 block of two pairs at once, on the upper triangle only: half
+//     the arithmetic of separate row and column passes over the whole matrix, and one barrier less.
+// The upper triangle of A (element type T, 8 bytes, odd pitch) lives in shared memory when it fits,
+// otherwise in the global workspace Wk.  The eigenvectors accumulate transposed in the global workspace
+// Vt (row k = eigenvector k): their update runs along contiguous rows, a warp per pair.
+// First Fock matrices of 256 alkanes (9 to 86 functions), double-float: 8.5 -> 5.8 ms; C2H6 / 6-31G* (42
+// functions), FP64: 2.6 -> 1.5 ms.
 template <typename T>
 __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, T* __restrict__ Vt_ws,
                                                 double* __restrict__ Vout, double* __restrict__ eps,
@@ -369,92 +400,126 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
 {
     extern __shared__ __align__(16) unsigned char jsm_raw[];
     __shared__ double red[32];
-    __shared__ int pp_[128], qq_[128];
-    __shared__ T cc_[128], ss_[128];
+    __shared__ unsigned char pp_[kJacMaxHalf], qq_[kJacMaxHalf], on_[kJacMaxHalf];
+    __shared__ __align__(16) unsigned char cc_raw[kJacMaxHalf * sizeof(T)], ss_raw[kJacMaxHalf * sizeof(T)];
     __shared__ int rotated;
+    T* cc_ = reinterpret_cast<T*>(cc_raw);
+    T* ss_ = reinterpret_cast<T*>(ss_raw);
+    typedef typename JacSum<T>::type Sum;
     const int m = blockIdx.x;
     if (!L.active[m]) return;
     const int n = L.n[m];
     const long long o = L.base[m];
+    const int pitch = use_smem ? (n | 1) : n;
     T* A = use_smem ? reinterpret_cast<T*>(jsm_raw) : Wk + o;
     T* Vt = Vt_ws + o;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
     const int npad = n + (n & 1), half = npad / 2, rounds = npad - 1;
-    const T one = jac_one<T>(), zero = jac_zero<T>();
-    double nrm = 0.0;
+    const int nblk = half * (half - 1) / 2;
+    const T one = jac_const<T>(1.0f), zero = jac_const<T>(0.0f);
+    Sum nrm = 0;
     for (int i = warp; i < n; i += nwarp)
         for (int j = lane; j < n; j += 32) {
-            jac_set(A[i * n + j], Ain[o + (long long)i * n + j]);
             Vt[i * n + j] = (i == j) ? one : zero;
-            const double a = jac_lead(A[i * n + j]);
-            nrm += a * a;
+            if (j < i) continue;
+            T v;
+            jac_set(v, Ain[o + (long long)i * n + j]);
+            A[i * pitch + j] = v;
+            nrm += i == j ? jac_sq(v) : 2 * jac_sq(v);
         }
-    nrm = block_sum(nrm, red);   // (synchronises the block)
+    const double norm2 = block_sum((double)nrm, red);   // (synchronises the block)
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
-        double off = 0.0;
+        Sum off = 0;
         for (int i = warp; i < n; i += nwarp)
-            for (int j = lane; j < n; j += 32) {
-                const double a = jac_lead(A[i * n + j]);
-                if (i != j) off += a * a;
-            }
-        off = block_sum(off, red);
-        if (off <= JacEps<T>::off * nrm || off == 0.0) break;
+            for (int j = i + 1 + lane; j < n; j += 32) off += 2 * jac_sq(A[i * pitch + j]);
+        const double off2 = block_sum((double)off, red);
+        if (off2 <= JacEps<T>::off * norm2 || off2 == 0.0) break;
         if (threadIdx.x == 0) rotated = 0;
         __syncthreads();
         for (int r = 0; r < rounds; ++r) {
+            // the rotations, and the diagonal blocks they act on
             for (int k = threadIdx.x; k < half; k += blockDim.x) {
                 int a, b2;
                 if (k == 0) { a = rounds; b2 = r; }
-                else { a = (r + k) % rounds; b2 = (r - k + rounds) % rounds; }
+                else {
+                    a = r + k;
+                    if (a >= rounds) a -= rounds;
+                    b2 = r - k;
+                    if (b2 < 0) b2 += rounds;
+                }
                 const int p = min(a, b2), q = max(a, b2);
                 T c = one, s = zero;
+                int on = 0;
                 if (q < n) {
-                    const T apq = A[p * n + q];
-                    const T app = A[p * n + p], aqq = A[q * n + q];
-                    const double lpq = fabs(jac_lead(apq));
+                    const T apq = A[p * pitch + q], app = A[p * pitch + p], aqq = A[q * pitch + q];
+                    const float fpq = jac_f32(apq);
                     // rotate unless a_pq is negligible against the diagonal (round-off level)
-                    if (lpq > 1e-300 && lpq > JacEps<T>::skip * sqrt(fabs(jac_lead(app)) * fabs(jac_lead(aqq)))) {
-                        const T tau = (aqq - app) / (apq + apq);
-                        T t;
-                        if (fabs(jac_lead(tau)) > 1e15) {
-                            t = one / (tau + tau);   // t -> 1/(2 tau); tau^2 would overflow FP32
-                        } else {
-                            const T den = jac_abs(tau) + jac_sqrt(one + tau * tau);
-                            t = (jac_lead(tau) >= 0.0 ? one : -one) / den;
-                        }
-                        c = one / jac_sqrt(one + t * t);
-                        s = t * c;
+                    if (fabsf(fpq) > 1e-35f && fabsf(fpq) > JacEps<T>::skip * sqrtf(fabsf(jac_f32(app))) * sqrtf(fabsf(jac_f32(aqq)))) {
+                        const float tau = __fdividef(0.5f * jac_f32(aqq - app), fpq), ta = fabsf(tau);
+                        const float t = copysignf(ta > 1e9f ? __fdividef(0.5f, ta) : 1.0f / (ta + sqrtf(fmaf(tau, tau, 1.0f))), tau);
+                        c = jac_cos(one, t);
+                        s = jac_scale(c, t);
+                        on = 1;
                         rotated = 1;
+                        // rows, then columns, of the 2 x 2 diagonal block
+                        const T r00 = jac_comb(c, app, -s, apq), r01 = jac_comb(c, apq, -s, aqq);
+                        const T r10 = jac_comb(s, app, c, apq), r11 = jac_comb(s, apq, c, aqq);
+                        A[p * pitch + p] = jac_comb(c, r00, -s, r01);
+                        A[p * pitch + q] = jac_comb(s, r00, c, r01);
+                        A[q * pitch + q] = jac_comb(s, r10, c, r11);
                     }
                 }
-                pp_[k] = p; qq_[k] = q; cc_[k] = c; ss_[k] = s;
+                pp_[k] = (unsigned char)p; qq_[k] = (unsigned char)min(q, 255); cc_[k] = c; ss_[k] = s;
+                on_[k] = (unsigned char)(q < n ? on : 2);      // 2: the pair of the padding index
             }
             __syncthreads();
-            // rows p, q:  row_p <- c row_p - s row_q,  row_q <- s row_p + c row_q  (a warp per pair)
-            for (int k = warp; k < half; k += nwarp) {
-                const int p = pp_[k], q = qq_[k];
-                if (q >= n || jac_iszero(ss_[k])) continue;
-                const T c = cc_[k], s = ss_[k];
-                for (int j = lane; j < n; j += 32) {
-                    const T x = A[p * n + j], y = A[q * n + j];
-                    A[p * n + j] = c * x - s * y;
-                    A[q * n + j] = s * x + c * y;
+            // the other 2 x 2 blocks (pair l > pair k), t = l (l - 1) / 2 + k
+            for (int t = threadIdx.x; t < nblk; t += blockDim.x) {
+                int l = (int)((1.0f + sqrtf(8.0f * (float)t + 1.0f)) * 0.5f);
+                while (l * (l - 1) / 2 > t) --l;
+                while ((l + 1) * l / 2 <= t) ++l;
+                const int k = t - l * (l - 1) / 2;
+                const int ok = on_[k], ol = on_[l];
+                if (!((ok | ol) & 1)) continue;
+                const int pk = pp_[k], qk = qq_[k], pl = pp_[l], ql = qq_[l];
+                T* const e0 = A + min(pk, pl) * pitch + max(pk, pl);
+                T* const e1 = ol == 2 ? e0 : A + min(pk, ql) * pitch + max(pk, ql);
+                T* const e2 = ok == 2 ? e0 : A + min(qk, pl) * pitch + max(qk, pl);
+                T* const e3 = ol == 2 ? e2 : (ok == 2 ? e1 : A + min(qk, ql) * pitch + max(qk, ql));
+                T x0 = *e0, x1 = *e1, x2 = *e2, x3 = *e3;
+                if (ok == 1) {
+                    const T c = cc_[k], s = ss_[k], ns = -s;
+                    const T y0 = jac_comb(c, x0, ns, x2), y1 = jac_comb(c, x1, ns, x3);
+                    x2 = jac_comb(s, x0, c, x2);
+                    x3 = jac_comb(s, x1, c, x3);
+                    x0 = y0;
+                    x1 = y1;
                 }
+                if (ol == 1) {
+                    const T c = cc_[l], s = ss_[l], ns = -s;
+                    const T y0 = jac_comb(c, x0, ns, x1), y2 = jac_comb(c, x2, ns, x3);
+                    x1 = jac_comb(s, x0, c, x1);
+                    x3 = jac_comb(s, x2, c, x3);
+                    x0 = y0;
+                    x2 = y2;
+                }
+                // a pair with the padding index has one row (or column): its other elements alias the first
+                if (ok != 2 && ol != 2) *e3 = x3;
+                if (ok != 2) *e2 = x2;
+                if (ol != 2) *e1 = x1;
+                *e0 = x0;
             }
-            __syncthreads();
-            // columns p, q of A; rows p, q of V^T
+            // rows p, q of V^T (a warp per pair)
             for (int k = warp; k < half; k += nwarp) {
-                const int p = pp_[k], q = qq_[k];
-                if (q >= n || jac_iszero(ss_[k])) continue;
-                const T c = cc_[k], s = ss_[k];
+                if (on_[k] != 1) continue;
+                T* const vp = Vt + pp_[k] * n;
+                T* const vq = Vt + qq_[k] * n;
+                const T c = cc_[k], s = ss_[k], ns = -s;
                 for (int i = lane; i < n; i += 32) {
-                    const T x = A[i * n + p], y = A[i * n + q];
-                    A[i * n + p] = c * x - s * y;
-                    A[i * n + q] = s * x + c * y;
-                    const T vx = Vt[p * n + i], vy = Vt[q * n + i];
-                    Vt[p * n + i] = c * vx - s * vy;
-                    Vt[q * n + i] = s * vx + c * vy;
+                    const T vx = vp[i], vy = vq[i];
+                    vp[i] = jac_comb(c, vx, ns, vy);
+                    vq[i] = jac_comb(s, vx, c, vy);
                 }
             }
             __syncthreads();
@@ -463,15 +528,16 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
         __syncthreads();
     }
     // eigenvalues ascending (rank by counting), eigenvectors (rows of V^T) into the columns of Vout
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double ai = jac_get(A[i * n + i]);
+    for (int i = warp; i < n; i += nwarp) {
+        const double ai = jac_get(A[i * pitch + i]);
         int rank = 0;
-        for (int j = 0; j < n; ++j) {
-            const double aj = jac_get(A[j * n + j]);
+        for (int j = lane; j < n; j += 32) {
+            const double aj = jac_get(A[j * pitch + j]);
             rank += (aj < ai) || (aj == ai && j < i);
         }
-        eps[ebase[m] + rank] = ai;
-        for (int r = 0; r < n; ++r) Vout[o + (long long)r * n + rank] = jac_get(Vt[i * n + r]);
+        for (int d = 16; d > 0; d >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, d);
+        if (lane == 0) eps[ebase[m] + rank] = ai;
+        for (int j = lane; j < n; j += 32) Vout[o + (long long)j * n + rank] = jac_get(Vt[i * n + j]);
     }
     if (threadIdx.x == 0 && sweeps_out) sweeps_out[m] = sweep;
 }
@@ -559,11 +625,13 @@ cudaError_t jacobi_prepare(SCFState& st)
 // workspaces W2 and Wk hold 8-byte elements of either type.
 cudaError_t jacobi(SCFState& st, const double* A, double* Vout, bool fp64 = true)
 {
+    // threads: a round updates about n^2 / 8 blocks of A and n^2 / 2 pairs of V's elements
+    const int threads = st.maxn <= 12 ? 64 : st.maxn <= 24 ? 128 : st.maxn <= 48 ? 256 : 512;
     if (fp64)
-        k_jacobi<double><<<st.nmol, 512, st.jac_smem, st.s>>>(A, st.W2.p, Vout, st.eps.p, st.ebase.p, st.L,
+        k_jacobi<double><<<st.nmol, threads, st.jac_smem, st.s>>>(A, st.W2.p, Vout, st.eps.p, st.ebase.p, st.L,
                                                               st.use_smem, st.Wk.p, 40, st.sweeps.p);
     else
-        k_jacobi<df32><<<st.nmol, 512, st.jac_smem, st.s>>>(A, reinterpret_cast<df32*>(st.W2.p), Vout, st.eps.p,
+        k_jacobi<df32><<<st.nmol, threads, st.jac_smem, st.s>>>(A, reinterpret_cast<df32*>(st.W2.p), Vout, st.eps.p,
                                                             st.ebase.p, st.L, st.use_smem,
                                                             reinterpret_cast<df32*>(st.Wk.p), 40, st.sweeps.p);
     return cudaGetLastError();
@@ -752,7 +820,7 @@ static mess_status scf_setup(SCFState& st, mess_basis* b, cudaStream_t caller, i
     }
     st.L = Layout{st.base.p, st.n.p, st.nocc.p, st.active.p, st.occ.p, st.ebase.p};
     // Jacobi matrix in shared memory when it fits
-    const size_t need = (size_t)st.maxn * st.maxn * sizeof(double);
+    const size_t need = (size_t)st.maxn * (st.maxn | 1) * sizeof(double);
     int dev = 0, smax = 0;
     MESS_CUDA_TRY(cudaGetDevice(&dev));
     MESS_CUDA_TRY(cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
