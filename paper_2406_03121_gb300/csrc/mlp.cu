@@ -217,82 +217,115 @@ __global__ void k_symmetrise(double* __restrict__ D, const long long* __restrict
 }
 
 // ------------------------------------------------------------------------------------ BF16 GEMM
-// C[m][n] (op)= sum_k A(m, k) B(k, n), A(m, k) = A[m * sam + k * sak], B(k, n) = B[k * sbk + n * sbn]
-// (BF16), FP32 accumulation on tensor cores (mma.sync m16n8k16).  64 x 64 block tile, 4 warps of
-// 32 x 32, K step 16.  gridDim.z splits K: slice z then stores its partial sums to part + z * pstride
-// (same layout as C), and k_sum_parts adds the slices in order z = 0, 1, ... (no atomics: training is
-// reproducible run to run).  Epilogue: + bias[n]; store FP32 to C (ldc) and optionally SiLU(C) as
-// BF16 to Abf (ldc).
+// C[m][n] = sum_k A(m, k) B(k, n) (BF16), FP32 accumulation on tensor cores (mma.sync m16n8k16).  AT: A
+// is stored k-major, A(m, k) = A[k * lda + m], else A[m * lda + k]; BT: B(k, n) = B[n * ldb + k], else
+// B[k * ldb + n].  Extents along the contiguous dimensions and the leading dimensions are multiples of 8
+// (16 bytes).  64 x 64 block tile, 4 warps of 32 x 32, K step 64 in two shared-memory stages filled by
+// 16-byte asynchronous copies, fragments by ldmatrix (transposing where the storage is).
+// gridDim.z splits K: slice z then stores its partial sums to part + z * pstride (same layout as C), and
+// k_sum_parts adds the slices in order z = 0, 1, ... (no atomics: training is reproducible run to run).
+// Epilogue, one of: + bias[n], C (ldc) as FP32 and SiLU(C) as BF16 to act (nullable); or, with dz, the
+// backward of SiLU: dz = BF16(sum * SiLU'(z)) only.
+// The matrices are small (K = 32 to 256 forward; 2048 rows, 16 blocks' worth of weight gradient), so the
+// kernel is bound by latency: filling stages by single elements took 320 us for a 256 x 256 weight gradient
+// over 2048 rows, now 6 us and the sum of its slices 11 us.  (tcgen05 would change the order of the FP32 sums, which the next
+// layer's BF16 rounding amplifies, and has nothing to gain at 0.1 % of the tensor peak.)
 struct GemmArgs {
     const __nv_bfloat16* A;
-    long long sam, sak;
+    long long lda;
     const __nv_bfloat16* B;
-    long long sbk, sbn;
+    long long ldb;
     float* C;
     long long ldc;
     const float* bias;
     __nv_bfloat16* act;     // SiLU(C + bias) as BF16 (nullable)
+    const float* z;         // with dz: pre-activation, same layout as C
+    __nv_bfloat16* dz;      // BF16(sum * SiLU'(z)) (nullable)
     int M, N, K;
+    int kchunk;             // K entries per slice
     float* part;            // split K: per-slice partial sums (no epilogue); null: one slice
     long long pstride;      // elements between slices of part
 };
 
-__device__ __forceinline__ unsigned pack2(__nv_bfloat16 lo, __nv_bfloat16 hi)
+constexpr int GT = 64, GP = GT + 8;   // tile side, shared-memory pitch (144 bytes: ldmatrix without conflicts)
+
+// a GT x GT tile of a matrix with `cols` contiguous entries per row (rows x cols from (r0, c0)), zero outside
+__device__ __forceinline__ void stage_tile(__nv_bfloat16* sm, const __nv_bfloat16* src, long long ld, int r0, int rows, int c0,
+                                           int cols)
 {
-    return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
+#pragma unroll
+    for (int i = 0; i < GT * GT / 8 / 128; ++i) {
+        const int t = (int)threadIdx.x + 128 * i, r = t / (GT / 8), c = (t % (GT / 8)) * 8;
+        const bool in = r0 + r < rows && c0 + c < cols;
+        const __nv_bfloat16* from = in ? src + (long long)(r0 + r) * ld + c0 + c : src;
+        const unsigned to = (unsigned)__cvta_generic_to_shared(sm + r * GP + c);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(to), "l"(from), "r"(in ? 16 : 0));
+    }
 }
 
-__global__ void __launch_bounds__(128) k_gemm_bf16(GemmArgs g)
+template <bool TRANS> __device__ __forceinline__ void load_matrices(unsigned (&f)[4], const __nv_bfloat16* at)
 {
-    __shared__ __nv_bfloat16 As[64][16 + 8];
-    __shared__ __nv_bfloat16 Bs[16][64 + 8];
+    const unsigned a = (unsigned)__cvta_generic_to_shared(at);
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(a));
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(f[0]), "=r"(f[1]), "=r"(f[2]), "=r"(f[3]) : "r"(a));
+}
+
+template <bool AT, bool BT> __global__ void __launch_bounds__(128) k_gemm_bf16(GemmArgs g)
+{
+    __shared__ __align__(16) __nv_bfloat16 As[2][GT * GP], Bs[2][GT * GP];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    const int kchunk = (g.K + gridDim.z - 1) / gridDim.z;
-    const int kbeg = blockIdx.z * kchunk, kend = min(g.K, kbeg + kchunk);
-    float acc[2][4][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-    const __nv_bfloat16 zero = __float2bfloat16(0.f);
-    for (int k0 = kbeg; k0 < kend; k0 += 16) {
-        for (int t = threadIdx.x; t < 64 * 16; t += 128) {
-            const int r = t / 16, c = t % 16;
-            const int gm = m0 + r, gk = k0 + c;
-            As[r][c] = (gm < g.M && gk < kend) ? g.A[(long long)gm * g.sam + (long long)gk * g.sak] : zero;
-        }
-        for (int t = threadIdx.x; t < 16 * 64; t += 128) {
-            const int r = t / 64, c = t % 64;
-            const int gk = k0 + r, gn = n0 + c;
-            Bs[r][c] = (gk < kend && gn < g.N) ? g.B[(long long)gk * g.sbk + (long long)gn * g.sbn] : zero;
+    const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
+    const int kbeg = blockIdx.z * g.kchunk, kend = min(g.K, kbeg + g.kchunk);
+    float acc[2][4][4] = {};
+    auto stage = [&](int st, int k0) {
+        if (AT) stage_tile(As[st], g.A, g.lda, k0, kend, m0, g.M);
+        else stage_tile(As[st], g.A, g.lda, m0, g.M, k0, kend);
+        if (BT) stage_tile(Bs[st], g.B, g.ldb, n0, g.N, k0, kend);
+        else stage_tile(Bs[st], g.B, g.ldb, k0, kend, n0, g.N);
+        asm volatile("cp.async.commit_group;\n");
+    };
+    const int mat = lane >> 3, r8 = lane & 7;
+    if (kbeg < kend) stage(0, kbeg);
+    for (int k0 = kbeg, st = 0; k0 < kend; k0 += GT, st ^= 1) {
+        if (k0 + GT < kend) {
+            stage(st ^ 1, k0 + GT);
+            asm volatile("cp.async.wait_group 1;\n");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n");
         }
         __syncthreads();
-        const int gid = lane >> 2, tig = lane & 3;
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            const int rb = wm + 16 * a;
-            unsigned af[4];
-            af[0] = pack2(As[rb + gid][tig * 2], As[rb + gid][tig * 2 + 1]);
-            af[1] = pack2(As[rb + gid + 8][tig * 2], As[rb + gid + 8][tig * 2 + 1]);
-            af[2] = pack2(As[rb + gid][tig * 2 + 8], As[rb + gid][tig * 2 + 9]);
-            af[3] = pack2(As[rb + gid + 8][tig * 2 + 8], As[rb + gid + 8][tig * 2 + 9]);
+        for (int kk = 0; kk < GT; kk += 16) {
+            unsigned af[2][4], bf[2][4];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int cb = wn + 8 * b;
-                unsigned bf[2];
-                bf[0] = pack2(Bs[tig * 2][cb + gid], Bs[tig * 2 + 1][cb + gid]);
-                bf[1] = pack2(Bs[tig * 2 + 8][cb + gid], Bs[tig * 2 + 9][cb + gid]);
-                float* c = acc[a][b];
-                asm volatile(
-                    "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                    "{%0,%1,%2,%3};\n"
-                    : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                    : "r"(af[0]), "r"(af[1]), "r"(af[2]), "r"(af[3]), "r"(bf[0]), "r"(bf[1]));
+            for (int a = 0; a < 2; ++a) {
+                // matrices in the order (m 0-7, k 0-7), (m 8-15, k 0-7), (m 0-7, k 8-15), (m 8-15, k 8-15)
+                const int mo = wm + 16 * a + (mat & 1) * 8, ko = kk + (mat >> 1) * 8;
+                load_matrices<AT>(af[a], AT ? &As[st][(ko + r8) * GP + mo] : &As[st][(mo + r8) * GP + ko]);
             }
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                // (k 0-7, n 0-7), (k 8-15, n 0-7), (k 0-7, n 8-15), (k 8-15, n 8-15)
+                const int no = wn + 16 * b + (mat >> 1) * 8, ko = kk + (mat & 1) * 8;
+                load_matrices<!BT>(bf[b], BT ? &Bs[st][(no + r8) * GP + ko] : &Bs[st][(ko + r8) * GP + no]);
+            }
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    float* c = acc[a][b];
+                    asm volatile(
+                        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                        "{%0,%1,%2,%3};\n"
+                        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                        : "r"(af[a][0]), "r"(af[a][1]), "r"(af[a][2]), "r"(af[a][3]), "r"(bf[b >> 1][2 * (b & 1)]),
+                          "r"(bf[b >> 1][2 * (b & 1) + 1]));
+                }
         }
         __syncthreads();
     }
@@ -306,12 +339,18 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(GemmArgs g)
                 const int r = m0 + wm + 16 * a + gid + (h >= 2 ? 8 : 0);
                 const int c = n0 + wn + 8 * b + tig * 2 + (h & 1);
                 if (r >= g.M || c >= g.N) continue;
+                const long long at = (long long)r * g.ldc + c;
                 float v = acc[a][b][h];
-                if (g.part) { g.part[blockIdx.z * g.pstride + (long long)r * g.ldc + c] = v; continue; }
-                float* dst = g.C + (long long)r * g.ldc + c;
+                if (g.part) { g.part[blockIdx.z * g.pstride + at] = v; continue; }
+                if (g.dz) {
+                    const float z = g.z[at];
+                    const float sg = 1.f / (1.f + __expf(-z));
+                    g.dz[at] = __float2bfloat16(v * sg * (1.f + z * (1.f - sg)));
+                    continue;
+                }
                 if (g.bias) v += g.bias[c];
-                *dst = v;
-                if (g.act) g.act[(long long)r * g.ldc + c] = __float2bfloat16(v / (1.f + __expf(-v)));
+                g.C[at] = v;
+                if (g.act) g.act[at] = __float2bfloat16(v / (1.f + __expf(-v)));
             }
 }
 
@@ -342,17 +381,6 @@ __global__ void k_loss(const float* __restrict__ Y, const float* __restrict__ T,
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv_count);
-}
-
-// dZ = dA * silu'(Z) as BF16, silu'(z) = s(z) (1 + z (1 - s(z))), s the logistic function
-__global__ void k_silu_back(const float* __restrict__ dA, const float* __restrict__ Z, __nv_bfloat16* __restrict__ dZ,
-                            long long n)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float z = Z[i];
-        const float sg = 1.f / (1.f + __expf(-z));
-        dZ[i] = __float2bfloat16(dA[i] * sg * (1.f + z * (1.f - sg)));
-    }
 }
 
 // out[i] = sum over slices z = 0 .. nz-1 (in that order) of part[z * pstride + i], for the M x N
@@ -418,7 +446,8 @@ struct mess_mlp {
     // activations of the current batch
     long long cap = 0;
     DevBuf<__nv_bfloat16> xb, a1, a2, dyb, dz2, dz1;
-    DevBuf<float> z1, z2, y, da2, da1;
+    DevBuf<float> z1, z2, y;
+    DevBuf<float> in;                           // X, T, M of mess_mlp_loss_grad (kept for repeated calls)
     DevBuf<double> loss;
     DevBuf<float> part;                         // per-slice partial sums of the gradient reductions
 };
@@ -438,8 +467,6 @@ cudaError_t ensure_cap(mess_mlp* m, long long rows)
     if ((e = m->z1.alloc(rows * WID)) != cudaSuccess) return e;
     if ((e = m->z2.alloc(rows * WID)) != cudaSuccess) return e;
     if ((e = m->y.alloc(rows * DOUT_PAD)) != cudaSuccess) return e;
-    if ((e = m->da2.alloc(rows * WID)) != cudaSuccess) return e;
-    if ((e = m->da1.alloc(rows * WID)) != cudaSuccess) return e;
     if (!m->part.p) {
         const long long most = std::max<long long>({(long long)WID * WID, (long long)DIN * WID, (long long)WID * DOUT_PAD});
         if ((e = m->part.alloc(MLP_MAX_SPLIT * most)) != cudaSuccess) return e;
@@ -450,20 +477,19 @@ cudaError_t ensure_cap(mess_mlp* m, long long rows)
 
 unsigned grid1(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 65535LL * 8); }
 
-cudaError_t gemm(const __nv_bfloat16* A, long long sam, long long sak, const __nv_bfloat16* B, long long sbk,
-                 long long sbn, float* C, long long ldc, int M, int N, int K, const float* bias,
-                 __nv_bfloat16* act, int splitk, cudaStream_t s, float* part = nullptr)
+// C = A B (+ bias, activations) with `split` slices of K; split > 1 only into the workspace of MLP_MAX_SPLIT
+// slices of M x ldc, then summed into C
+template <bool AT, bool BT> cudaError_t gemm(GemmArgs g, int split, cudaStream_t s, float* part = nullptr)
 {
-    // split K only into a workspace of MLP_MAX_SPLIT slices of M x ldc (no epilogue then)
-    if (splitk > 1 && (!part || splitk > MLP_MAX_SPLIT || bias || act)) return cudaErrorInvalidValue;
-    const long long pstride = (long long)M * ldc;
-    GemmArgs g{A, sam, sak, B, sbk, sbn, C, ldc, bias, act, M, N, K, splitk > 1 ? part : nullptr, pstride};
-    dim3 grid((N + 63) / 64, (M + 63) / 64, splitk);
-    k_gemm_bf16<<<grid, 128, 0, s>>>(g);
-    if (splitk > 1) k_sum_parts<<<grid1((long long)M * N), 256, 0, s>>>(part, splitk, pstride, M, N, ldc, C);
+    g.pstride = (long long)g.M * g.ldc;
+    g.kchunk = ((g.K + split - 1) / split + 15) / 16 * 16;
+    split = (g.K + g.kchunk - 1) / g.kchunk;
+    if (split > 1 && (!part || split > MLP_MAX_SPLIT || g.bias || g.act || g.dz)) return cudaErrorInvalidValue;
+    if (split > 1) g.part = part;
+    k_gemm_bf16<AT, BT><<<dim3((g.N + GT - 1) / GT, (g.M + GT - 1) / GT, split), 128, 0, s>>>(g);
+    if (split > 1) k_sum_parts<<<grid1((long long)g.M * g.N), 256, 0, s>>>(part, split, g.pstride, g.M, g.N, g.ldc, g.C);
     return cudaGetLastError();
 }
-
 
 // forward of `rows` rows whose FP32 descriptors are in X (device); output Y (rows x 32, FP32)
 cudaError_t forward(mess_mlp* m, const float* X, long long rows, cudaStream_t s)
@@ -473,12 +499,16 @@ cudaError_t forward(mess_mlp* m, const float* X, long long rows, cudaStream_t s)
     const __nv_bfloat16* wb = m->wb.p;
     k_to_bf16<<<grid1(rows * DIN), 256, 0, s>>>(X, m->xb.p, rows * DIN);
     const float* w = m->w.p;
-    if ((e = gemm(m->xb.p, DIN, 1, wb + MlpParams::W1, WID, 1, m->z1.p, WID, (int)rows, WID, DIN,
-                  w + MlpParams::B1, m->a1.p, 1, s)) != cudaSuccess) return e;
-    if ((e = gemm(m->a1.p, WID, 1, wb + MlpParams::W2, WID, 1, m->z2.p, WID, (int)rows, WID, WID,
-                  w + MlpParams::B2, m->a2.p, 1, s)) != cudaSuccess) return e;
-    return gemm(m->a2.p, WID, 1, wb + MlpParams::W3, DOUT_PAD, 1, m->y.p, DOUT_PAD, (int)rows, DOUT_PAD, WID,
-                w + MlpParams::B3, nullptr, 1, s);
+    auto layer = [&](const __nv_bfloat16* in, int k, int w_off, int n, int b_off, float* z, __nv_bfloat16* act) {
+        GemmArgs g{};
+        g.A = in; g.lda = k; g.B = wb + w_off; g.ldb = n; g.C = z; g.ldc = n;
+        g.bias = w + b_off; g.act = act;
+        g.M = (int)rows; g.N = n; g.K = k;
+        return gemm<false, false>(g, 1, s);
+    };
+    if ((e = layer(m->xb.p, DIN, MlpParams::W1, WID, MlpParams::B1, m->z1.p, m->a1.p)) != cudaSuccess) return e;
+    if ((e = layer(m->a1.p, WID, MlpParams::W2, WID, MlpParams::B2, m->z2.p, m->a2.p)) != cudaSuccess) return e;
+    return layer(m->a2.p, WID, MlpParams::W3, DOUT_PAD, MlpParams::B3, m->y.p, nullptr);
 }
 
 // loss and gradient (into m->g) of the rows forward() just processed
@@ -490,30 +520,36 @@ cudaError_t backward(mess_mlp* m, const float* T, const float* M, long long rows
     k_loss<<<grid1(rows * DOUT_PAD), 256, 0, s>>>(m->y.p, T, M, rows, 1.0 / std::max(1.0, count), m->loss.p, m->dyb.p);
     const __nv_bfloat16* wb = m->wb.p;
     float* g = m->g.p;
-    const int split = (int)std::min<long long>(MLP_MAX_SPLIT, std::max<long long>(1, rows / 4096));
+    // weight gradients: 16 tiles at most, so K (the rows) is split until about two blocks per SM work on
+    // them, 64 rows (one stage) or more each; the slices are summed in order
+    const int split = (int)std::min<long long>(24, std::max<long long>(1, rows / 64));
     float* part = m->part.p;
     auto colsum = [&](const __nv_bfloat16* X, int cols, float* out) {
         k_colsum<<<dim3((cols + 31) / 32, MLP_MAX_SPLIT), 256, 0, s>>>(X, rows, cols, part);
         k_sum_parts<<<grid1(cols), 256, 0, s>>>(part, MLP_MAX_SPLIT, cols, 1, cols, cols, out);
     };
-    // layer 3: dW3 = A2^T dY, db3 = sum dY, dA2 = dY W3^T
-    if ((e = gemm(m->a2.p, 1, WID, m->dyb.p, DOUT_PAD, 1, g + MlpParams::W3, DOUT_PAD, WID, DOUT_PAD, (int)rows,
-                  nullptr, nullptr, split, s, part)) != cudaSuccess) return e;
-    colsum(m->dyb.p, DOUT_PAD, g + MlpParams::B3);
-    if ((e = gemm(m->dyb.p, DOUT_PAD, 1, wb + MlpParams::W3, 1, DOUT_PAD, m->da2.p, WID, (int)rows, WID, DOUT_PAD,
-                  nullptr, nullptr, 1, s)) != cudaSuccess) return e;
-    k_silu_back<<<grid1(rows * WID), 256, 0, s>>>(m->da2.p, m->z2.p, m->dz2.p, rows * WID);
-    // layer 2
-    if ((e = gemm(m->a1.p, 1, WID, m->dz2.p, WID, 1, g + MlpParams::W2, WID, WID, WID, (int)rows,
-                  nullptr, nullptr, split, s, part)) != cudaSuccess) return e;
-    colsum(m->dz2.p, WID, g + MlpParams::B2);
-    if ((e = gemm(m->dz2.p, WID, 1, wb + MlpParams::W2, 1, WID, m->da1.p, WID, (int)rows, WID, WID,
-                  nullptr, nullptr, 1, s)) != cudaSuccess) return e;
-    k_silu_back<<<grid1(rows * WID), 256, 0, s>>>(m->da1.p, m->z1.p, m->dz1.p, rows * WID);
-    // layer 1
-    if ((e = gemm(m->xb.p, 1, DIN, m->dz1.p, WID, 1, g + MlpParams::W1, WID, DIN, WID, (int)rows,
-                  nullptr, nullptr, split, s, part)) != cudaSuccess) return e;
-    colsum(m->dz1.p, WID, g + MlpParams::B1);
+    // dW = in^T dout, db = column sums of dout
+    auto weights = [&](const __nv_bfloat16* in, int k, const __nv_bfloat16* dout, int n, int w_off, int b_off) {
+        GemmArgs a{};
+        a.A = in; a.lda = k; a.B = dout; a.ldb = n; a.C = g + w_off; a.ldc = n;
+        a.M = k; a.N = n; a.K = (int)rows;
+        const cudaError_t r = gemm<true, false>(a, split, s, part);
+        if (r == cudaSuccess) colsum(dout, n, g + b_off);
+        return r;
+    };
+    // d(pre-activation of the layer below) = (dout W^T) SiLU'(z)
+    auto below = [&](const __nv_bfloat16* dout, int n, int w_off, const float* z, __nv_bfloat16* dz) {
+        GemmArgs a{};
+        a.A = dout; a.lda = n; a.B = wb + w_off; a.ldb = n; a.ldc = WID;
+        a.z = z; a.dz = dz;
+        a.M = (int)rows; a.N = WID; a.K = n;
+        return gemm<false, true>(a, 1, s);
+    };
+    if ((e = weights(m->a2.p, WID, m->dyb.p, DOUT_PAD, MlpParams::W3, MlpParams::B3)) != cudaSuccess) return e;
+    if ((e = below(m->dyb.p, DOUT_PAD, MlpParams::W3, m->z2.p, m->dz2.p)) != cudaSuccess) return e;
+    if ((e = weights(m->a1.p, WID, m->dz2.p, WID, MlpParams::W2, MlpParams::B2)) != cudaSuccess) return e;
+    if ((e = below(m->dz2.p, WID, MlpParams::W2, m->z1.p, m->dz1.p)) != cudaSuccess) return e;
+    if ((e = weights(m->xb.p, DIN, m->dz1.p, WID, MlpParams::W1, MlpParams::B1)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -612,7 +648,7 @@ mess_status init_params(mess_mlp* m, unsigned long long seed)
 
 void free_mlp(mess_mlp* m)
 {
-    for (DevBuf<float>* d : {&m->w, &m->g, &m->m1, &m->m2, &m->z1, &m->z2, &m->y, &m->da2, &m->da1}) d->free();
+    for (DevBuf<float>* d : {&m->w, &m->g, &m->m1, &m->m2, &m->z1, &m->z2, &m->y, &m->in}) d->free();
     for (DevBuf<__nv_bfloat16>* d : {&m->wb, &m->xb, &m->a1, &m->a2, &m->dyb, &m->dz2, &m->dz1}) d->free();
     m->loss.free();
 }
@@ -760,17 +796,16 @@ extern "C" mess_status mess_mlp_loss_grad(mess_mlp* m, long long nrows, const fl
                                           double* loss, float* grad)
 {
     if (!m || !X || !T || !M || nrows <= 0) { mess_set_error("bad arguments"); return MESS_EINVAL; }
-    DevBuf<float> dX, dT, dM;
-    MESS_CUDA_TRY(dX.alloc(nrows * DIN));
-    MESS_CUDA_TRY(dT.alloc(nrows * DOUT));
-    MESS_CUDA_TRY(dM.alloc(nrows * DOUT));
-    MESS_CUDA_TRY(cudaMemcpy(dX.p, X, sizeof(float) * nrows * DIN, cudaMemcpyHostToDevice));
-    MESS_CUDA_TRY(cudaMemcpy(dT.p, T, sizeof(float) * nrows * DOUT, cudaMemcpyHostToDevice));
-    MESS_CUDA_TRY(cudaMemcpy(dM.p, M, sizeof(float) * nrows * DOUT, cudaMemcpyHostToDevice));
-    double count = 0.0;
-    for (long long i = 0; i < nrows * DOUT; ++i) count += M[i];
-    MESS_CUDA_TRY(forward(m, dX.p, nrows, 0));
-    MESS_CUDA_TRY(backward(m, dT.p, dM.p, nrows, count, 0));
+    const size_t nx = (size_t)nrows * DIN, nt = (size_t)nrows * DOUT;
+    if (m->in.n < nx + 2 * nt) MESS_CUDA_TRY(m->in.alloc(nx + 2 * nt));
+    float *dX = m->in.p, *dT = dX + nx, *dM = dT + nt;
+    MESS_CUDA_TRY(cudaMemcpy(dX, X, sizeof(float) * nx, cudaMemcpyHostToDevice));
+    MESS_CUDA_TRY(forward(m, dX, nrows, 0));
+    double count = 0.0;                            // (while the forward pass runs)
+    for (size_t i = 0; i < nt; ++i) count += M[i];
+    MESS_CUDA_TRY(cudaMemcpy(dT, T, sizeof(float) * nt, cudaMemcpyHostToDevice));
+    MESS_CUDA_TRY(cudaMemcpy(dM, M, sizeof(float) * nt, cudaMemcpyHostToDevice));
+    MESS_CUDA_TRY(backward(m, dT, dM, nrows, count, 0));
     MESS_CUDA_TRY(cudaDeviceSynchronize());
     if (loss) MESS_CUDA_TRY(cudaMemcpy(loss, m->loss.p, sizeof(double), cudaMemcpyDeviceToHost));
     if (grad) MESS_CUDA_TRY(cudaMemcpy(grad, m->g.p, sizeof(float) * MlpParams::N, cudaMemcpyDeviceToHost));
