@@ -178,7 +178,7 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
     B.parts.clear();
     // per ket list (pair class x primitive group): Q, and prefix sums of unique function pairs and of
     // primitive pairs, in list order
-    const int NL = MESS_NUM_PCLASS * MESS_NGROUP;
+    const int NL = MESS_NLIST;
     std::vector<std::vector<long long>> fpre_l(NL), ppre_l(NL);
     for (int Lk = 0; Lk < NL; ++Lk) {
         const std::vector<int>& kl = b->class_list[Lk];
@@ -197,24 +197,25 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
     // within one pair class); each builds its parts (FP64-class / reduced-precision split) into its
     // own arrays.  Tasks are independent and run on host threads; the parts are concatenated in task
     // order, so the bins do not depend on the threading.
-    struct Task { int p1, p2, g1, g2; std::vector<BinPart> parts; std::vector<int> bra, kbeg; std::vector<long long> offs; };
+    struct Task { int p1, p2, L1, L2; std::vector<BinPart> parts; std::vector<int> bra, kbeg; std::vector<long long> offs; };
     std::vector<Task> tasks;
     for (int p1 = 0; p1 < MESS_NUM_PCLASS; ++p1)
         for (int p2 = 0; p2 <= p1; ++p2)
-            for (int g1 = 0; g1 < MESS_NGROUP; ++g1)
-                for (int g2 = 0; g2 < MESS_NGROUP; ++g2) {
-                    if (p1 == p2 && g2 > g1) continue;
-                    if (b->class_list[p1 * MESS_NGROUP + g1].empty() || b->class_list[p2 * MESS_NGROUP + g2].empty()) continue;
-                    tasks.push_back(Task{p1, p2, g1, g2, {}, {}, {}, {}});
+            for (int h1 = 0; h1 < 2 * MESS_NGROUP; ++h1)
+                for (int h2 = 0; h2 < 2 * MESS_NGROUP; ++h2) {
+                    const int x1 = h1 / MESS_NGROUP, x2 = h2 / MESS_NGROUP;   // pairs with an extra shell
+                    if ((p1 == p2 && h2 > h1) || (x1 && x2)) continue;
+                    const int L1 = MESS_LIST(x1, p1, h1 % MESS_NGROUP), L2 = MESS_LIST(x2, p2, h2 % MESS_NGROUP);
+                    if (b->class_list[L1].empty() || b->class_list[L2].empty()) continue;
+                    tasks.push_back(Task{p1, p2, L1, L2, {}, {}, {}, {}});
                 }
     auto run_task = [&](Task& T) {
-        const int p1 = T.p1, p2 = T.p2, g1 = T.g1, g2 = T.g2;
-        const int L1 = p1 * MESS_NGROUP + g1, L2 = p2 * MESS_NGROUP + g2;
+        const int p1 = T.p1, p2 = T.p2, L1 = T.L1, L2 = T.L2;
         const std::vector<int>& bl = b->class_list[L1];
         const std::vector<long long>& fpre = fpre_l[L2];
         const std::vector<long long>& ppre = ppre_l[L2];
         const std::vector<int>& kl = b->class_list[L2];
-        const bool same = p1 == p2 && g1 == g2;
+        const bool same = L1 == L2;
         std::vector<int>& bra = T.bra;
         std::vector<int>& kbeg = T.kbeg;
         std::vector<long long>& offs = T.offs;
@@ -529,7 +530,7 @@ static mess_status build_pairs(mess_basis* b)
                     const HostShell& sa = b->shells[A];
                     const HostShell& sb = b->shells[B];
                     const bool canonical = sa.l > sb.l || (sa.l == sb.l && A >= B);
-                    if (!canonical) continue;
+                    if (!canonical || (A >= b->first_extra && B >= b->first_extra)) continue;
                     c.pa.push_back(A);
                     c.pb.push_back(B);
                     c.pcls.push_back(pclass_of(sa.l, sb.l));
@@ -730,6 +731,30 @@ static mess_status build_pairs(mess_basis* b)
     return MESS_OK;
 }
 
+// Pair lists (MESS_LIST): per molecule, pairs sorted by Q descending
+static mess_status build_lists(mess_basis* b)
+{
+    std::vector<std::vector<std::vector<int>>> per(MESS_NLIST, std::vector<std::vector<int>>(b->nmol));
+    for (int p = 0; p < b->npair; ++p)
+        per[MESS_LIST(b->extra(p) ? 1 : 0, b->pair_class[p], prim_group(b->pp_n[p]))][b->pair_mol[p]].push_back(p);
+    for (int L = 0; L < MESS_NLIST; ++L) {
+        std::vector<int> l;
+        std::vector<int> seg(1, 0);
+        for (int m = 0; m < b->nmol; ++m) {
+            std::stable_sort(per[L][m].begin(), per[L][m].end(), [&](int x, int y) { return b->Q[x] > b->Q[y]; });
+            l.insert(l.end(), per[L][m].begin(), per[L][m].end());
+            seg.push_back((int)l.size());
+        }
+        b->class_list[L] = l;
+        b->class_seg[L] = seg;
+        MESS_CUDA_TRY(b->d_class_list[L].upload(l));
+        std::vector<KetRec> rl(l.size());
+        for (size_t k = 0; k < l.size(); ++k) rl[k] = b->pair_rec[l[k]];
+        MESS_CUDA_TRY(b->d_ketrec[L].upload(rl));
+    }
+    return MESS_OK;
+}
+
 static mess_status build_schwarz(mess_basis* b)
 {
     std::vector<int> lists[MESS_NUM_PCLASS];
@@ -761,29 +786,7 @@ static mess_status build_schwarz(mess_basis* b)
         MESS_CUDA_TRY(b->d_Qf.upload(qf));
         b->P64.Qf = b->P32.Qf = b->Pdf.Qf = b->d_Qf.p;
     }
-    // lists per (class, primitive-count group): per molecule, pairs sorted by Q descending
-    for (int c = 0; c < MESS_NUM_PCLASS; ++c) {
-        for (int g = 0; g < MESS_NGROUP; ++g) {
-            std::vector<std::vector<int>> per(b->nmol);
-            for (int p : lists[c])
-                if (prim_group(b->pp_n[p]) == g) per[b->pair_mol[p]].push_back(p);
-            std::vector<int> l;
-            std::vector<int> seg(1, 0);
-            for (int m = 0; m < b->nmol; ++m) {
-                std::stable_sort(per[m].begin(), per[m].end(), [&](int x, int y) { return b->Q[x] > b->Q[y]; });
-                l.insert(l.end(), per[m].begin(), per[m].end());
-                seg.push_back((int)l.size());
-            }
-            const int L = c * MESS_NGROUP + g;
-            b->class_list[L] = l;
-            b->class_seg[L] = seg;
-            MESS_CUDA_TRY(b->d_class_list[L].upload(l));
-            std::vector<KetRec> rl(l.size());
-            for (size_t k = 0; k < l.size(); ++k) rl[k] = b->pair_rec[l[k]];
-            MESS_CUDA_TRY(b->d_ketrec[L].upload(rl));
-        }
-    }
-    return MESS_OK;
+    return build_lists(b);
 }
 
 void mess_free_basis(mess_basis* b)
@@ -873,8 +876,11 @@ mess_status mess_derivative_basis(const mess_basis* b, mess_basis** out, std::ve
     mess_basis* e = new (std::nothrow) mess_basis();
     if (!e) { mess_set_error("host allocation failed"); return MESS_ENOMEM; }
     add_molecule(e, b->Z, b->xyz, sh);
+    e->first_extra = ns;
     mess_status st = build_pairs(e);
-    if (st == MESS_OK) st = build_schwarz(e);
+    // its builds are not screened: no Schwarz factors (the lists keep the order of the pairs)
+    e->Q.assign(e->npair, 0.0);
+    if (st == MESS_OK) st = build_lists(e);
     if (st != MESS_OK) { mess_free_basis(e); delete e; return st; }
     e->gpu_ready = true;
     *out = e;

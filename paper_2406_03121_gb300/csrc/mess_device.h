@@ -34,6 +34,10 @@
 #define MESS_LMAX 2               // s, p, Cartesian d
 #define MESS_NUM_PCLASS 6         // pair classes (la,lb): ss ps pp ds dp dd
 #define MESS_NGROUP 3             // primitive-pair count groups: <= 3, 4..12, >= 13
+// pair lists: per class, primitive group and whether the pair has an extra shell (a raised or lowered
+// shell of a derivative basis; none elsewhere)
+#define MESS_NLIST (2 * MESS_NUM_PCLASS * MESS_NGROUP)
+#define MESS_LIST(extra, pclass, group) (((extra) * MESS_NUM_PCLASS + (pclass)) * MESS_NGROUP + (group))
 #define MESS_TEAM_WARPS 4         // warps (one shell quartet each) per block of the large-class kernels
 
 // One primitive pair: zeta, PAx, PAy, PAz (P - A, P the Gaussian product centre), K, 1/(2 zeta), and

@@ -140,12 +140,17 @@ struct mess_basis {
     int npair = 0;
     std::vector<int> pair_a, pair_b, pair_class, pp_off, pp_n, pair_mol;
     std::vector<double> Q;          // Schwarz factor per pair
-    // pair lists per (pair class c, primitive-count group g) at index c * MESS_NGROUP + g: pair ids,
-    // per molecule sorted by Q descending, with nmol + 1 segment offsets
-    std::vector<int> class_list[MESS_NUM_PCLASS * MESS_NGROUP];
-    std::vector<int> class_seg[MESS_NUM_PCLASS * MESS_NGROUP];
-    DevBuf<int> d_class_list[MESS_NUM_PCLASS * MESS_NGROUP];
-    DevBuf<KetRec> d_ketrec[MESS_NUM_PCLASS * MESS_NGROUP];   // the lists' pair records, list order
+    // pair lists at MESS_LIST(extra, pair class, primitive-count group): pair ids, per molecule sorted by Q
+    // descending, with nmol + 1 segment offsets
+    std::vector<int> class_list[MESS_NLIST];
+    std::vector<int> class_seg[MESS_NLIST];
+    DevBuf<int> d_class_list[MESS_NLIST];
+    DevBuf<KetRec> d_ketrec[MESS_NLIST];    // the lists' pair records, list order
+    // shells from this index on are extra (derivative bases: the raised and lowered shells after the
+    // molecule's own).  A pair has at most one of them, and so has a quartet: the gradient's J', K' need no
+    // others.  (All: none is extra.)
+    int first_extra = 0x7fffffff;
+    bool extra(int pair) const { return pair_a[pair] >= first_extra || pair_b[pair] >= first_extra; }
     std::vector<KetRec> pair_rec;                             // per pair
     DevBuf<KetRec> d_pair_rec;
 

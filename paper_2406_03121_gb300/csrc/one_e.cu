@@ -107,7 +107,7 @@ __host__ __device__ constexpr int binom(int n, int k) { return k == 0 || k == n 
 template <int N> __device__ __forceinline__ double ipow(double x) { return N == 0 ? 1.0 : (N == 1 ? x : x * x); }
 
 struct Seg { const int* list; int count, block0, la, lb; };   // pairs of one class and primitive group
-constexpr int kMaxSeg = MESS_NUM_PCLASS * MESS_NGROUP;
+constexpr int kMaxSeg = MESS_NLIST;
 
 struct OneEArgs {
     Seg seg[kMaxSeg];
@@ -281,8 +281,8 @@ cudaError_t mess_launch_one_e(const mess_basis* b, double* dS, double* dT, doubl
     int blocks = 0;
     // the longest pairs first: dd to ss, many primitives to few
     for (int c = MESS_NUM_PCLASS - 1; c >= 0; --c)
-        for (int g = MESS_NGROUP - 1; g >= 0; --g) {
-            const DevBuf<int>& l = b->d_class_list[c * MESS_NGROUP + g];
+        for (int g = 2 * MESS_NGROUP - 1; g >= 0; --g) {
+            const DevBuf<int>& l = b->d_class_list[MESS_LIST(g / MESS_NGROUP, c, g % MESS_NGROUP)];
             if (l.n == 0) continue;
             s.seg[s.nseg++] = Seg{l.p, (int)l.n, blocks, cls[c][0], cls[c][1]};
             blocks += ((int)l.n + kPairsPerBlock - 1) / kPairsPerBlock;
