@@ -114,9 +114,9 @@ struct JKGraph {
 struct XcState {
     bool ready = false;
     long long npts = 0, ao = 0, mol_npts_max = 0;
-    DevBuf<double> pts, w, phi, dphi, vrho, vgrad, Exc;
-    DevBuf<int> atom, mol, fbase, shell_off, shell_n, shell_fl;
-    DevBuf<long long> pbase, aobase;
+    DevBuf<double> pts, w, phi, dphi, vrho, vgrad, Exc, tab;
+    DevBuf<int> atom, atom_mol, radial_at, radial_n, fbase, shell_off, shell_n, shell_fl;
+    DevBuf<long long> pbase, aobase, abase;
 };
 
 // A basis of one molecule, or (internally) of a batch of molecules: shells, pairs and quartets

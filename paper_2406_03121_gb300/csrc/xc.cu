@@ -68,12 +68,37 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w)
 }
 
 // ------------------------------------------------------------------------------------------ kernels
+// Points and weights before the partition, one thread per point.  tab: the angular table (cos theta,
+// sin theta, weight for kNTheta; cos phi, sin phi for kNPhi), then per radial grid its radii and weights.
+// (Tabulated on the host and copied, the 3.3 million points of 64 H2 took about 70 ms of a call; here 0.05.)
+constexpr int kAngular = kNTheta * kNPhi, kAngularTab = 3 * kNTheta + 2 * kNPhi;
+constexpr int kRadialMax = 75, kGridThreads = 256, kBlocksPerAtom = kRadialMax * kAngular / kGridThreads;
+static_assert(kRadialMax * kAngular % kGridThreads == 0, "whole blocks per atom");
+
+__global__ void __launch_bounds__(kGridThreads) k_grid(const double* __restrict__ tab, const int* __restrict__ radial_at,
+                                                       const int* __restrict__ radial_n, const long long* __restrict__ abase,
+                                                       const double* __restrict__ xyz, double* __restrict__ pts,
+                                                       double* __restrict__ w, int* __restrict__ atom)
+{
+    const int A = blockIdx.x / kBlocksPerAtom;
+    const int t = (blockIdx.x % kBlocksPerAtom) * kGridThreads + threadIdx.x;
+    const int i = t / kAngular, th = t % kAngular / kNPhi, ph = t % kNPhi, nr = radial_n[A];
+    if (i >= nr) return;
+    const double* rad = tab + radial_at[A];
+    const double r = rad[i], st = tab[kNTheta + th];
+    const long long p = abase[A] + t;
+    pts[3 * p] = xyz[3 * A] + r * st * tab[3 * kNTheta + ph];
+    pts[3 * p + 1] = xyz[3 * A + 1] + r * st * tab[3 * kNTheta + kNPhi + ph];
+    pts[3 * p + 2] = xyz[3 * A + 2] + r * tab[th];
+    w[p] = rad[nr + i] * tab[2 * kNTheta + th] * 2.0 * M_PI / kNPhi;
+    atom[p] = A;
+}
+
 struct GridArgs {
     const double* pts;       // [npts][3]
     double* w;               // [npts] radial x angular weight, times the partition after k_becke
     const int* atom;         // [npts] global atom index of the point's atomic grid
-    const int* mol;          // [npts]
-    const long long* pbase;  // [nmol + 1] first point of each molecule
+    const int* atom_mol;     // [natom]
     const int* atom_off;     // [nmol] first atom of each molecule
     const int* atom_n;       // [nmol]
     const double* xyz;       // [natom][3]
@@ -84,7 +109,7 @@ __global__ void k_becke(GridArgs g)
 {
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= g.npts) return;
-    const int m = g.mol[p], a0 = g.atom_off[m], na = g.atom_n[m], own = g.atom[p];
+    const int own = g.atom[p], m = g.atom_mol[own], a0 = g.atom_off[m], na = g.atom_n[m];
     if (na == 1) return;
     const double x = g.pts[3 * p], y = g.pts[3 * p + 1], z = g.pts[3 * p + 2];
     double sum = 0.0, mine = 0.0;
@@ -110,7 +135,8 @@ __global__ void k_becke(GridArgs g)
 
 struct AoArgs {
     const double* pts;
-    const int* mol;
+    const int* atom;         // [npts]
+    const int* atom_mol;     // [natom]
     long long npts;
     const int* shell_off;    // [nmol] first shell of the molecule
     const int* shell_n;      // [nmol]
@@ -137,7 +163,7 @@ __global__ void k_ao(AoArgs a)
 {
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.npts) return;
-    const int m = a.mol[p], n = a.mn[m];
+    const int m = a.atom_mol[a.atom[p]], n = a.mn[m];
     const long long lp = p - a.pbase[m], np_ = a.pbase[m + 1] - a.pbase[m];
     double* ph = a.phi + a.aobase[m] + lp;
     double* dx = a.dphi + 3 * a.aobase[m] + lp;
@@ -455,7 +481,8 @@ __global__ void __launch_bounds__(kVxcThreads) k_vxc(VxcArgs v)
 void mess_free_xc(mess_basis* b)
 {
     XcState& x = b->xc;
-    x.pts.free(); x.w.free(); x.atom.free(); x.mol.free(); x.pbase.free(); x.phi.free(); x.dphi.free();
+    x.pts.free(); x.w.free(); x.atom.free(); x.atom_mol.free(); x.tab.free(); x.radial_at.free(); x.radial_n.free();
+    x.abase.free(); x.pbase.free(); x.phi.free(); x.dphi.free();
     x.aobase.free(); x.vrho.free(); x.vgrad.free(); x.fbase.free(); x.shell_off.free(); x.shell_n.free();
     x.shell_fl.free(); x.Exc.free();
     x.npts = 0;
@@ -466,53 +493,67 @@ mess_status mess_xc_prepare(mess_basis* b, cudaStream_t s)
 {
     XcState& X = b->xc;
     if (X.ready) return MESS_OK;
-    std::vector<double> pts, w;
-    std::vector<int> atom, mol;
-    std::vector<long long> pbase(1, 0), aobase;
-    std::vector<double> ct, wt;
-    gauss_legendre(kNTheta, ct, wt);
-    long long ao = 0;
-    for (int m = 0; m < b->nmol; ++m) {
-        const long long start = (long long)w.size();
-        for (int A = b->mol_atom_off[m]; A < b->mol_atom_off[m] + b->mol_atom_n[m]; ++A) {
-            const int Z = b->Z[A];
-            const int nr = Z == 1 ? 50 : 75;
-            const double R = radius_of(Z) * kAngstrom;
-            for (int i = 1; i <= nr; ++i) {
-                const double th = i * M_PI / (nr + 1);
-                const double xr = cos(th);
-                const double wx = M_PI / (nr + 1) * sin(th) * sin(th) / sqrt(1.0 - xr * xr);
-                const double r = R * (1.0 + xr) / (1.0 - xr);
-                const double wr = wx * r * r * 2.0 * R / ((1.0 - xr) * (1.0 - xr));
-                for (int t = 0; t < kNTheta; ++t) {
-                    const double st = sqrt(1.0 - ct[t] * ct[t]);
-                    for (int k = 0; k < kNPhi; ++k) {
-                        const double ph = 2.0 * M_PI * k / kNPhi;
-                        pts.push_back(b->xyz[3 * A] + r * st * cos(ph));
-                        pts.push_back(b->xyz[3 * A + 1] + r * st * sin(ph));
-                        pts.push_back(b->xyz[3 * A + 2] + r * ct[t]);
-                        w.push_back(wr * wt[t] * 2.0 * M_PI / kNPhi);
-                        atom.push_back(A);
-                        mol.push_back(m);
-                    }
-                }
-            }
+    // angular table, then the radial grid of every element present
+    std::vector<double> tab((size_t)kAngularTab);
+    {
+        std::vector<double> ct, wt;
+        gauss_legendre(kNTheta, ct, wt);
+        for (int t = 0; t < kNTheta; ++t) {
+            tab[t] = ct[t];
+            tab[kNTheta + t] = sqrt(1.0 - ct[t] * ct[t]);
+            tab[2 * kNTheta + t] = wt[t];
         }
-        pbase.push_back((long long)w.size());
+        for (int k = 0; k < kNPhi; ++k) {
+            tab[3 * kNTheta + k] = cos(2.0 * M_PI * k / kNPhi);
+            tab[3 * kNTheta + kNPhi + k] = sin(2.0 * M_PI * k / kNPhi);
+        }
+    }
+    std::vector<int> at_of_z(128, -1), radial_at(b->natom), radial_n(b->natom), atom_mol(b->natom);
+    std::vector<long long> pbase(1, 0), aobase, abase(b->natom);
+    long long ao = 0, np = 0;
+    for (int m = 0; m < b->nmol; ++m) {
+        const long long start = np;
+        for (int A = b->mol_atom_off[m]; A < b->mol_atom_off[m] + b->mol_atom_n[m]; ++A) {
+            const int Z = b->Z[A], nr = Z == 1 ? 50 : kRadialMax;
+            if (at_of_z[Z] < 0) {
+                at_of_z[Z] = (int)tab.size();
+                const double R = radius_of(Z) * kAngstrom;
+                std::vector<double> rw;
+                for (int i = 1; i <= nr; ++i) {
+                    const double th = i * M_PI / (nr + 1);
+                    const double xr = cos(th);
+                    const double wx = M_PI / (nr + 1) * sin(th) * sin(th) / sqrt(1.0 - xr * xr);
+                    const double r = R * (1.0 + xr) / (1.0 - xr);
+                    tab.push_back(r);
+                    rw.push_back(wx * r * r * 2.0 * R / ((1.0 - xr) * (1.0 - xr)));
+                }
+                tab.insert(tab.end(), rw.begin(), rw.end());
+            }
+            radial_at[A] = at_of_z[Z];
+            radial_n[A] = nr;
+            atom_mol[A] = m;
+            abase[A] = np;
+            np += (long long)nr * kAngular;
+        }
+        pbase.push_back(np);
         aobase.push_back(ao);
-        ao += ((long long)w.size() - start) * b->mol_nbf[m];
+        ao += (np - start) * b->mol_nbf[m];
     }
     std::vector<int> fbase(b->nmol, 0), shell_fl;
     for (int m = 1; m < b->nmol; ++m) fbase[m] = fbase[m - 1] + b->mol_nbf[m - 1];
     for (const HostShell& sh : b->shells) shell_fl.push_back(sh.fl);
-    X.npts = (long long)w.size();
+    X.npts = np;
     X.ao = ao;
     X.mol_npts_max = 0;
     for (int m = 0; m < b->nmol; ++m) X.mol_npts_max = std::max(X.mol_npts_max, pbase[m + 1] - pbase[m]);
-    MESS_CUDA_TRY(X.pts.upload(pts));
-    MESS_CUDA_TRY(X.w.upload(w));
-    MESS_CUDA_TRY(X.atom.upload(atom));
-    MESS_CUDA_TRY(X.mol.upload(mol));
+    MESS_CUDA_TRY(X.tab.upload(tab));
+    MESS_CUDA_TRY(X.radial_at.upload(radial_at));
+    MESS_CUDA_TRY(X.radial_n.upload(radial_n));
+    MESS_CUDA_TRY(X.atom_mol.upload(atom_mol));
+    MESS_CUDA_TRY(X.abase.upload(abase));
+    MESS_CUDA_TRY(X.pts.alloc((size_t)np * 3));
+    MESS_CUDA_TRY(X.w.alloc((size_t)np));
+    MESS_CUDA_TRY(X.atom.alloc((size_t)np));
     MESS_CUDA_TRY(X.pbase.upload(pbase));
     MESS_CUDA_TRY(X.aobase.upload(aobase));
     MESS_CUDA_TRY(X.fbase.upload(fbase));
@@ -526,10 +567,13 @@ mess_status mess_xc_prepare(mess_basis* b, cudaStream_t s)
     MESS_CUDA_TRY(X.Exc.alloc((size_t)b->nmol));
     const int T = 256;
     const unsigned blocks = (unsigned)((X.npts + T - 1) / T);
-    GridArgs g{X.pts.p, X.w.p, X.atom.p, X.mol.p, X.pbase.p, b->d_mol_atom_off.p, b->d_mol_atom_n.p, b->d_xyz.p, X.npts};
+    k_grid<<<(unsigned)(b->natom * kBlocksPerAtom), kGridThreads, 0, s>>>(X.tab.p, X.radial_at.p, X.radial_n.p, X.abase.p,
+                                                                          b->d_xyz.p, X.pts.p, X.w.p, X.atom.p);
+    MESS_CUDA_TRY(cudaGetLastError());
+    GridArgs g{X.pts.p, X.w.p, X.atom.p, X.atom_mol.p, b->d_mol_atom_off.p, b->d_mol_atom_n.p, b->d_xyz.p, X.npts};
     k_becke<<<blocks, T, 0, s>>>(g);
     MESS_CUDA_TRY(cudaGetLastError());
-    AoArgs a{X.pts.p, X.mol.p, X.npts, X.shell_off.p, X.shell_n.p, b->d_shell_l.p, b->d_shell_K.p, b->d_shell_poff.p,
+    AoArgs a{X.pts.p, X.atom.p, X.atom_mol.p, X.npts, X.shell_off.p, X.shell_n.p, b->d_shell_l.p, b->d_shell_K.p, b->d_shell_poff.p,
              X.shell_fl.p, b->d_shell_R.p, b->d_shell_alpha.p, b->d_shell_coef.p, b->d_fscale.p, X.fbase.p, X.pbase.p,
              X.aobase.p, b->d_mol_n.p, X.phi.p, X.dphi.p};
     k_ao<<<blocks, T, 0, s>>>(a);
