@@ -681,6 +681,21 @@ def df32_program(info):
     return info["mode"] == "straight" and info["vrr_flops"] + info["hrr_flops"] >= 250
 
 
+def line_types(info):
+    """Arithmetic types whose one-thread kernel runs straight-line code in a class.  The straight classes:
+    all, but double-float in the larger ones (df32_program).  The op-program classes: FP32 up to 324
+    integrals and FP64 up to 162 - the compiler keeps those in registers with a few KB of spills, and a
+    quartet then takes a tenth of the instructions of the interpreter (a warp per quartet); beyond, it
+    gives up on registers."""
+    if info["mode"] == "straight":
+        return ("float", "double") if df32_program(info) else ("float", "double", "df32")
+    return tuple(t for t, most in (("float", 324), ("double", 162)) if info["nint"] <= most)
+
+
+def is_type(types):
+    return " || ".join(f"std::is_same<R, {t}>::value" for t in types)
+
+
 def emit_class(cls):
     body, info = emit_class_straight(cls)
     (la, lb), (lc, ld) = cls
@@ -711,7 +726,10 @@ def emit_class(cls):
     pr = build_program(cls)
     info["mode"] = "program"
     info["nv_slots"], info["nh_slots"] = pr["nv"], pr["nh"]
+    types = line_types(info)
     L = []
+    if types:
+        L.append(body.replace(f"__device__ __forceinline__ void eri_{t}(", f"__device__ __forceinline__ void eri_{t}_sl(", 1))
     L.append(f"// ---- class ({la}{lb}|{lc}{ld}): op program, {len(pr['vrr'])} VRR ops on {pr['nv']} slots, "
              f"{len(pr['hrr'])} HRR ops on {pr['nh']} slots")
     L += emit_program_tables(t, pr)
@@ -720,6 +738,9 @@ def emit_class(cls):
     L.append("{")
     L.append("    static_assert(G == 1, \"op-program classes run one thread per quartet\");")
     L.append("    (void)g; (void)sh;")
+    if types:
+        L.append(f"    if constexpr ({is_type(types)}) eri_{t}_sl<R, BMODE, G>(P, bp, kv, g, I, live);")
+        L.append("    else")
     L.append(f"    eri_program<R, BMODE, {pr['L']}, {pr['nv']}, {pr['nh']}, {pr['nacc']}, {len(pr['vrr'])}, "
              f"{len(pr['hrr'])}, {len(pr['fin'])}>(P, bp, kv, vprog_{t}, hprog_{t}, fslot_{t}, fscale_{t}, "
              f"fscaleh_{t}, fscalel_{t}, I, live);")
@@ -792,12 +813,24 @@ def team_capable(info):
 
 def emit_digests(cls, info):
     """The digestion of a class as the kernels call it (digest_<class>).  Straight-line classes stage
-    the density blocks in registers; the op-program classes, and the double-float path of the
+    the density blocks in registers.  The op-program classes, and the double-float path of the
     straight-line classes that run the interpreter (df32_program), read D through the read-only
-    cache: a one-thread kernel that inlines the interpreter must not also stage density arrays."""
+    cache: a one-thread kernel that inlines the interpreter must not also stage density arrays.  Where
+    the one-thread kernel of an op-program class is straight-line code (line_types) its loops are
+    unrolled, so that the integrals need not be indexed in local memory."""
     t = tag(cls)
     if info["mode"] != "straight":
-        return emit_digest(cls, unroll=False)
+        types = line_types(info)
+        if not types:
+            return emit_digest(cls, unroll=False)
+        return (emit_digest(cls, unroll=True, stage=False, name=f"digest_{t}_ul") + "\n"
+                + emit_digest(cls, unroll=False, name=f"digest_{t}_ro") + "\n"
+                + "template <typename R>\n"
+                + f"__device__ __forceinline__ void digest_{t}(const R* I, const DigestCtx<R>& c, R s)\n"
+                + "{\n"
+                + f"    if constexpr ({is_type(types)}) digest_{t}_ul<R>(I, c, s);\n"
+                + f"    else digest_{t}_ro<R>(I, c, s);\n"
+                + "}\n")
     if not df32_program(info):
         return emit_digest(cls, unroll=True)
     return (emit_digest(cls, unroll=True, name=f"digest_{t}_st") + "\n"
@@ -810,10 +843,12 @@ def emit_digests(cls, info):
             + "}\n")
 
 
-def emit_digest(cls, unroll=True, name=None):
+def emit_digest(cls, unroll=True, name=None, stage=None):
     """J/K digestion of one shell quartet (see the kernel file for the accumulation convention).
-    unroll=True: density blocks staged in registers, loops fully unrolled (small classes);
-    unroll=False: compact loops reading the density through the read-only cache (large classes)."""
+    unroll=True: loops fully unrolled, density blocks staged in registers (small classes; stage=False: read
+    where they are used); unroll=False: compact loops reading the density through the read-only cache
+    (large classes)."""
+    stage = unroll if stage is None else stage
     (la, lb), (lc, ld) = cls
     t = tag(cls)
     na, nb, nc, nd = ncart(la), ncart(lb), ncart(lc), ncart(ld)
@@ -827,7 +862,7 @@ def emit_digest(cls, unroll=True, name=None):
               ("Dbc", ("c.fb", nb), ("c.fc", nc)), ("Dbd", ("c.fb", nb), ("c.fd", nd)))
     dref = {}
     for nm, (r0, nr), (c0, ncol) in blocks:
-        if unroll:
+        if stage:
             L.append(f"    R {nm}[{nr * ncol}];")
             L.append(PR)
             L.append(f"    for (int i = 0; i < {nr}; ++i)")
@@ -1011,16 +1046,18 @@ def main(outdir):
     # class table (host + device readable)
     tab = ["// Generated by gen_eri.py: do not edit.", "#pragma once", "",
            f"#define MESS_NUM_QCLASS {len(QUARTET_CLASSES)}", "",
-           "// straight: straight-line kernels with G = 1, 4, 8 lanes per quartet (else one op-program",
-           "// kernel, G = 1); team: a warp-per-quartet kernel exists",
-           "typedef struct { int la, lb, lc, ld, L, nint, nacc, nvrr; long vrr_flops, hrr_flops; int straight, team; }",
+           "// straight: kernels with G = 1, 4, 8, 32 lanes per quartet (else G = 1 only); team: a",
+           "// warp-per-quartet kernel exists; line: the one-thread kernel is straight-line code (else the op",
+           "// program) in FP32 (1), FP64 (2), double-float (4)",
+           "typedef struct { int la, lb, lc, ld, L, nint, nacc, nvrr; long vrr_flops, hrr_flops; int straight, team, line; }",
            "    mess_qclass_info;",
            "static const mess_qclass_info MESS_QCLASS[MESS_NUM_QCLASS] = {"]
     for f in infos:
         st = 1 if f["mode"] == "straight" else 0
         tm = 1 if (team_capable(f) or f["mode"] == "program") else 0
+        ln = sum({"float": 1, "double": 2, "df32": 4}[x] for x in line_types(f))
         tab.append(f"    {{{f['la']}, {f['lb']}, {f['lc']}, {f['ld']}, {f['L']}, {f['nint']}, {f['nacc']}, "
-                   f"{f['nvrr']}, {f['vrr_flops']}, {f['hrr_flops']}, {st}, {tm}}},")
+                   f"{f['nvrr']}, {f['vrr_flops']}, {f['hrr_flops']}, {st}, {tm}, {ln}}},")
     tab.append("};")
     text = "\n".join(tab) + "\n"
     path = os.path.join(outdir, "eri_classes.h")
