@@ -20,6 +20,7 @@
 #include <cuda_profiler_api.h>
 #include <cstdlib>
 
+#include "jk_cost.h"
 #include "mess_internal.h"
 
 // ------------------------------------------------------------------------------------------ errors
@@ -271,23 +272,6 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
             }
             bp.nbra = (int)bra.size() - bp.bra_off;
             offs.push_back(bp.total);
-            // heavily contracted quartets: split the primitive loop over 8 lanes
-            const bool straight = MESS_QCLASS[bp.qclass].straight != 0;
-            const double avg = bp.total > 0 ? (double)bp.prim_quartets / (double)bp.total : 0.0;
-            // lanes per quartet (the choice when the kernels are not autotuned).  FP64-class parts: 8 for
-            // long primitive loops, 4 for medium loops of parts too small to fill the GPU one thread per
-            // quartet.  Reduced-precision parts: one thread per quartet unless the part is small and its
-            // loops long - with G lanes only one lane in G digests, and for the small classes the
-            // digestion is most of the per-quartet work (measured on STO-3G alkanes, 81 primitive
-            // quartets per shell quartet: one thread per quartet 2.2x faster than 8 lanes).
-            if (!straight) bp.G = 1;
-            else if (fp64) bp.G = avg >= 24.0 ? 8 : ((avg >= 6.0 && bp.total < (1LL << 18)) ? 4 : 1);
-            else bp.G = (avg >= 6.0 && bp.total < (1LL << 15)) ? 4 : 1;
-            // warp per quartet: always for the op-program classes; for small FP64 parts of the classes
-            // with at least 40 VRR entries (too few quartets to fill the GPU one thread each:
-            // measured better below about 2e6 quartets x VRR entries, worse above)
-            const double work = (double)bp.total * MESS_QCLASS[bp.qclass].nvrr;
-            bp.team = (!straight || (fp64 && MESS_QCLASS[bp.qclass].team && bp.G == 1 && work < 2e6)) ? 1 : 0;
             if (bp.nbra > 0) T.parts.push_back(bp);
             else offs.resize(bp.offs_off);
         }
@@ -1052,6 +1036,28 @@ static int part_mode(const BinPart& p, const mess_jk_opts& o)
     return o.boys_fp64 ? MESS_MODE_MIXED : MESS_MODE_FP32;
 }
 
+static JkWork part_work(const BinPart& p)
+{
+    const mess_qclass_info& c = MESS_QCLASS[p.qclass];
+    double fp, fs;
+    class_flops(p.qclass, &fp, &fs);
+    return JkWork{fp, (double)c.hrr_flops + c.nacc, 12.0 * c.nint, (double)p.total, (double)p.prim_quartets};
+}
+
+// Kernel shape of every part of the bins under these options: as set by the caller or the autotuner, else
+// the one that jk_cost.h picks.
+static std::vector<JkShape> part_shapes(const mess_basis* b, const mess_jk_opts& o)
+{
+    const std::vector<BinPart>& parts = b->bins.parts;
+    std::vector<JkShape> shape(parts.size());
+    for (size_t k = 0; k < parts.size(); ++k) {
+        const BinPart& p = parts[k];
+        const int mode = part_mode(p, o);
+        shape[k] = p.fixed ? JkShape{p.G, p.team, mode} : jk_choose(MESS_QCLASS[p.qclass], mode, part_work(p));
+    }
+    return shape;
+}
+
 // The launches of one J/K build, all on stream s or forked from it onto the pool's streams and
 // joined back: zero J and K, convert D for the reduced-precision parts, one launch per bin part
 // (most expensive first), symmetrise.  With parts != null every launch runs on s between timing
@@ -1069,30 +1075,33 @@ static mess_status jk_enqueue(mess_basis* b, const mess_jk_opts& o, const double
                                                   b->packed, s));
         inf.kernel_launches += 1;
     }
-    // launch order: most expensive parts first (FP64, then by algorithmic work)
+    // launch order: the parts estimated longest first, each on the stream with the least estimated work
+    // so far (a long serial chain then starts at once and has a stream to itself)
     std::vector<size_t> order(b->bins.parts.size());
     std::iota(order.begin(), order.end(), (size_t)0);
-    auto cost = [&](const BinPart& p) {
-        double fp, fs;
-        class_flops(p.qclass, &fp, &fs);
-        return (fp * (double)p.prim_quartets + fs * (double)p.total) * (p.fp64 ? 62.0 : 1.0);
-    };
-    std::stable_sort(order.begin(), order.end(),
-                     [&](size_t x, size_t y) { return cost(b->bins.parts[x]) > cost(b->bins.parts[y]); });
+    const std::vector<JkShape> shape = part_shapes(b, o);
+    std::vector<double> us(order.size());
+    for (size_t k = 0; k < order.size(); ++k)
+        us[k] = jk_time(MESS_QCLASS[b->bins.parts[k].qclass], shape[k], part_work(b->bins.parts[k]));
+    std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return us[x] > us[y]; });
     const bool concurrent = pool != nullptr;
     if (concurrent) {
         MESS_CUDA_TRY(cudaEventRecord(pool->fork, s));
         for (int i = 0; i < pool->n; ++i) MESS_CUDA_TRY(cudaStreamWaitEvent(pool->s[i], pool->fork, 0));
     }
     mess_status out = MESS_OK;
-    for (size_t r = 0; r < order.size(); ++r) {
-        const size_t k = order[r];
+    double load[MESS_MAX_STREAMS] = {};
+    for (size_t k : order) {
         const BinPart& p = b->bins.parts[k];
+        int lane = 0;
+        for (int i = 1; concurrent && i < pool->n; ++i)
+            if (load[i] < load[lane]) lane = i;
+        load[lane] += us[k];
         ClassLaunchArgs a{};
         a.kind = MESS_KIND_JK;
-        a.mode = part_mode(p, o);
-        a.G = p.G;
-        a.team = p.team;
+        a.mode = shape[k].mode;
+        a.G = shape[k].G;
+        a.team = shape[k].team;
         a.bin = bin_launch(b, p);
         a.P64_ptr = &b->P64;
         a.P32_ptr = &b->P32;
@@ -1103,7 +1112,7 @@ static mess_status jk_enqueue(mess_basis* b, const mess_jk_opts& o, const double
         a.J = dJ;
         a.K = dK;
         a.n = b->nbf;
-        a.stream = concurrent ? pool->s[r % pool->n] : s;
+        a.stream = concurrent ? pool->s[lane] : s;
         if (ev) cudaEventRecord((*ev)[2 * k], s);
         cudaError_t e = MESS_CLASS_LAUNCHERS[p.qclass](a);
         if (ev) cudaEventRecord((*ev)[2 * k + 1], s);
@@ -1233,6 +1242,7 @@ static mess_status jk_run(mess_basis* b, const double* dD, double* dJ, double* d
             cudaError_t e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) { mess_set_error("profile sync: %s", cudaGetErrorString(e)); out = MESS_ECUDA; }
         }
+        const std::vector<JkShape> shape = part_shapes(b, o);
         for (size_t k = 0; out == MESS_OK && k < b->bins.parts.size(); ++k) {
             const BinPart& p = b->bins.parts[k];
             const mess_qclass_info& c = MESS_QCLASS[p.qclass];
@@ -1243,9 +1253,9 @@ static mess_status jk_run(mess_basis* b, const double* dD, double* dJ, double* d
             r.shell_quartets = p.total;
             r.primitive_quartets = p.prim_quartets;
             r.function_quartets = p.fn_quartets;
-            r.G = p.G;
-            r.team = p.team;
-            r.mode = part_mode(p, o);
+            r.G = shape[k].G;
+            r.team = shape[k].team;
+            r.mode = shape[k].mode;
             double fp, fs;
             class_flops(p.qclass, &fp, &fs);
             r.flops = fp * (double)p.prim_quartets + fs * (double)p.total;
@@ -1387,7 +1397,8 @@ static mess_status jk_autotune_device(mess_basis* b, const double* dD, double* d
     MESS_CUDA_TRY(cudaEventCreate(&e0));
     cudaError_t ce = cudaEventCreate(&e1);
     if (ce != cudaSuccess) { cudaEventDestroy(e0); mess_set_error("%s", cudaGetErrorString(ce)); return MESS_ECUDA; }
-    struct Variant { int G, team, mode; };
+    const std::vector<JkShape> shape = part_shapes(b, o);   // before tuning
+    size_t part_no = 0;
     int changed = 0;
     mess_status out = MESS_OK;
     for (BinPart& p : b->bins.parts) {
@@ -1399,7 +1410,7 @@ static mess_status jk_autotune_device(mess_basis* b, const double* dD, double* d
         } else {
             modes.push_back(o.boys_fp64 ? MESS_MODE_MIXED : MESS_MODE_FP32);
         }
-        std::vector<Variant> cand;
+        std::vector<JkShape> cand;
         for (int m : modes) {
             if (c.straight) {
                 cand.push_back({1, 0, m});
@@ -1415,10 +1426,10 @@ static mess_status jk_autotune_device(mess_basis* b, const double* dD, double* d
                 cand.push_back({1, 3, m});
             }
         }
-        const Variant before{p.G, p.team, part_mode(p, o)};
-        Variant best = before;
+        const JkShape before = shape[part_no++];
+        JkShape best = before;
         float best_ms = 3.4e38f;
-        for (const Variant& v : cand) {
+        for (const JkShape& v : cand) {
             ClassLaunchArgs a{};
             a.kind = MESS_KIND_JK;
             a.mode = v.mode;
@@ -1471,7 +1482,7 @@ static mess_status jk_autotune_device(mess_basis* b, const double* dD, double* d
         p.G = best.G;
         p.team = best.team;
         p.mode = best.mode;
-        p.tuned = 1;
+        p.fixed = 1;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1504,14 +1515,16 @@ extern "C" mess_status mess_jk_set_variant(const mess_basis* bc, const mess_jk_o
         return MESS_EINVAL;
     }
     int changed = 0;
-    for (BinPart& p : b->bins.parts) {
+    const std::vector<JkShape> shape = part_shapes(b, o);
+    for (size_t k = 0; k < b->bins.parts.size(); ++k) {
+        BinPart& p = b->bins.parts[k];
         const mess_qclass_info& c = MESS_QCLASS[p.qclass];
-        const int G0 = p.G, t0 = p.team, m0 = part_mode(p, o);
         if (!c.straight) { p.G = 1; p.team = team; }                  // op-program classes: G = 1 only
         else if (team && c.team) { p.team = team; p.G = 1; }
         else { p.team = 0; p.G = G; }
         if (p.fp64 && split_mode >= 0) p.mode = split_mode;
-        if (p.G != G0 || p.team != t0 || part_mode(p, o) != m0) ++changed;
+        p.fixed = 1;
+        if (p.G != shape[k].G || p.team != shape[k].team || part_mode(p, o) != shape[k].mode) ++changed;
     }
     b->bins.generation += 1;
     mess_free_jk_graphs(b);
@@ -1535,12 +1548,12 @@ extern "C" mess_status mess_jk_get_tuning(const mess_basis* bc, const mess_jk_op
     *nparts = np;
     if (!table) return MESS_OK;
     if (max_parts < np) { mess_set_error("mess_jk_get_tuning: %d parts, max_parts = %d", np, max_parts); return MESS_EINVAL; }
+    const std::vector<JkShape> shape = part_shapes(b, o);
     for (int k = 0; k < np; ++k) {
-        const BinPart& p = b->bins.parts[k];
-        table[4 * k] = p.qclass;
-        table[4 * k + 1] = p.G;
-        table[4 * k + 2] = p.team;
-        table[4 * k + 3] = part_mode(p, o);
+        table[4 * k] = b->bins.parts[k].qclass;
+        table[4 * k + 1] = shape[k].G;
+        table[4 * k + 2] = shape[k].team;
+        table[4 * k + 3] = shape[k].mode;
     }
     return MESS_OK;
 }
@@ -1573,7 +1586,7 @@ extern "C" mess_status mess_jk_set_tuning(const mess_basis* bc, const mess_jk_op
         p.G = table[4 * k + 1];
         p.team = table[4 * k + 2];
         p.mode = table[4 * k + 3];
-        p.tuned = 1;
+        p.fixed = 1;
     }
     b->bins.generation += 1;
     mess_free_jk_graphs(b);
