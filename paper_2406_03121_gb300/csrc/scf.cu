@@ -381,17 +381,18 @@ constexpr int kJacMaxHalf = 128;   // pairs of a round (n <= 256)
 // rotation of (p, q) uses tau = (a_qq - a_pp)/(2 a_pq), t = sign(tau)/(|tau| + sqrt(1 + tau^2)),
 // c = 1/sqrt(1 + t^2), s = t c, and A <- J^T A J, V <- V J.  Eigenvalues ascending in eps, the
 // matching eigenvectors as the columns of Vout.
-// A round is bound by its serial chain (rotation angles, barrier, update, barrier) for small matrices
-// and by the instructions of the update for large ones (FP64: the FP64 pipe), so:
+// A round is bound by its serial chains (rotation angles, the update of A, memory latency of V) and, in
+// FP64, by the FP64 pipe of the one SM, so:
 //   - t is taken in FP32 (a rotation by a slightly wrong angle is still a rotation: it leaves 1e-7 of a_pq
 //     for the next sweep); c and s have c^2 + s^2 = 1 to the accuracy of T;
 //   - both sides of the update act on the 2 x 2 block of two pairs at once, on the upper triangle only: half
-//     the arithmetic of separate row and column passes over the whole matrix, and one barrier less.
+//     the arithmetic of separate row and column passes over the whole matrix;
+//   - the angles of the next round are found by one to four warps while the others update V.
 // The upper triangle of A (element type T, 8 bytes, odd pitch) lives in shared memory when it fits,
 // otherwise in the global workspace Wk.  The eigenvectors accumulate transposed in the global workspace
-// Vt (row k = eigenvector k): their update runs along contiguous rows, a warp per pair.
-// First Fock matrices of 256 alkanes (9 to 86 functions), double-float: 8.5 -> 5.8 ms; C2H6 / 6-31G* (42
-// functions), FP64: 2.6 -> 1.5 ms.
+// Vt (row k = eigenvector k): their update runs along contiguous rows, four elements in flight per thread.
+// First Fock matrices of 256 alkanes (9 to 86 functions), double-float: 8.5 -> 5.5 ms (5.8 with
+// the angles found between the rounds); C2H6 / 6-31G* (42 functions), FP64: 2.6 -> 1.1 ms (1.5).
 template <typename T>
 __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, T* __restrict__ Vt_ws,
                                                 double* __restrict__ Vout, double* __restrict__ eps,
@@ -400,11 +401,9 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
 {
     extern __shared__ __align__(16) unsigned char jsm_raw[];
     __shared__ double red[32];
-    __shared__ unsigned char pp_[kJacMaxHalf], qq_[kJacMaxHalf], on_[kJacMaxHalf];
-    __shared__ __align__(16) unsigned char cc_raw[kJacMaxHalf * sizeof(T)], ss_raw[kJacMaxHalf * sizeof(T)];
+    __shared__ unsigned char pp2[2][kJacMaxHalf], qq2[2][kJacMaxHalf], on2[2][kJacMaxHalf];   // (round parity)
+    __shared__ __align__(16) unsigned char cc_raw[2 * kJacMaxHalf * sizeof(T)], ss_raw[2 * kJacMaxHalf * sizeof(T)];
     __shared__ int rotated;
-    T* cc_ = reinterpret_cast<T*>(cc_raw);
-    T* ss_ = reinterpret_cast<T*>(ss_raw);
     typedef typename JacSum<T>::type Sum;
     const int m = blockIdx.x;
     if (!L.active[m]) return;
@@ -417,6 +416,51 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
     const int npad = n + (n & 1), half = npad / 2, rounds = npad - 1;
     const int nblk = half * (half - 1) / 2;
     const T one = jac_const<T>(1.0f), zero = jac_const<T>(0.0f);
+    // threads of the V update: all but the warps that find the angles
+    const int nvt = (int)blockDim.x - (half + 31) / 32 * 32, vthread = (int)threadIdx.x - ((int)blockDim.x - nvt);
+    const int vdk = nvt / n, vdi = nvt % n;
+    // the rotations of round r, and the diagonal blocks they act on: one pair per thread
+    auto rotations = [&](int r) {
+        const int par = r & 1;
+        if (threadIdx.x < half) {
+            const int k = threadIdx.x;
+            int a, b2;
+            if (k == 0) { a = rounds; b2 = r; }
+            else {
+                a = r + k;
+                if (a >= rounds) a -= rounds;
+                b2 = r - k;
+                if (b2 < 0) b2 += rounds;
+            }
+            const int p = min(a, b2), q = max(a, b2);
+            T c = one, s = zero;
+            int on = 0;
+            if (q < n) {
+                const T apq = A[p * pitch + q], app = A[p * pitch + p], aqq = A[q * pitch + q];
+                const float fpq = jac_f32(apq);
+                // rotate unless a_pq is negligible against the diagonal (round-off level)
+                if (fabsf(fpq) > 1e-35f && fabsf(fpq) > JacEps<T>::skip * sqrtf(fabsf(jac_f32(app))) * sqrtf(fabsf(jac_f32(aqq)))) {
+                    const float tau = __fdividef(0.5f * jac_f32(aqq - app), fpq), ta = fabsf(tau);
+                    const float t = copysignf(ta > 1e9f ? __fdividef(0.5f, ta) : 1.0f / (ta + sqrtf(fmaf(tau, tau, 1.0f))), tau);
+                    c = jac_cos(one, t);
+                    s = jac_scale(c, t);
+                    on = 1;
+                    rotated = 1;
+                    // rows, then columns, of the 2 x 2 diagonal block
+                    const T r00 = jac_comb(c, app, -s, apq), r01 = jac_comb(c, apq, -s, aqq);
+                    const T r10 = jac_comb(s, app, c, apq), r11 = jac_comb(s, apq, c, aqq);
+                    A[p * pitch + p] = jac_comb(c, r00, -s, r01);
+                    A[p * pitch + q] = jac_comb(s, r00, c, r01);
+                    A[q * pitch + q] = jac_comb(s, r10, c, r11);
+                }
+            }
+            pp2[par][k] = (unsigned char)p;
+            qq2[par][k] = (unsigned char)min(q, 255);
+            reinterpret_cast<T*>(cc_raw)[par * kJacMaxHalf + k] = c;
+            reinterpret_cast<T*>(ss_raw)[par * kJacMaxHalf + k] = s;
+            on2[par][k] = (unsigned char)(q < n ? on : 2);      // 2: the pair of the padding index
+        }
+    };
     Sum nrm = 0;
     for (int i = warp; i < n; i += nwarp)
         for (int j = lane; j < n; j += 32) {
@@ -437,43 +481,12 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
         if (off2 <= JacEps<T>::off * norm2 || off2 == 0.0) break;
         if (threadIdx.x == 0) rotated = 0;
         __syncthreads();
+        rotations(0);
+        __syncthreads();
         for (int r = 0; r < rounds; ++r) {
-            // the rotations, and the diagonal blocks they act on
-            for (int k = threadIdx.x; k < half; k += blockDim.x) {
-                int a, b2;
-                if (k == 0) { a = rounds; b2 = r; }
-                else {
-                    a = r + k;
-                    if (a >= rounds) a -= rounds;
-                    b2 = r - k;
-                    if (b2 < 0) b2 += rounds;
-                }
-                const int p = min(a, b2), q = max(a, b2);
-                T c = one, s = zero;
-                int on = 0;
-                if (q < n) {
-                    const T apq = A[p * pitch + q], app = A[p * pitch + p], aqq = A[q * pitch + q];
-                    const float fpq = jac_f32(apq);
-                    // rotate unless a_pq is negligible against the diagonal (round-off level)
-                    if (fabsf(fpq) > 1e-35f && fabsf(fpq) > JacEps<T>::skip * sqrtf(fabsf(jac_f32(app))) * sqrtf(fabsf(jac_f32(aqq)))) {
-                        const float tau = __fdividef(0.5f * jac_f32(aqq - app), fpq), ta = fabsf(tau);
-                        const float t = copysignf(ta > 1e9f ? __fdividef(0.5f, ta) : 1.0f / (ta + sqrtf(fmaf(tau, tau, 1.0f))), tau);
-                        c = jac_cos(one, t);
-                        s = jac_scale(c, t);
-                        on = 1;
-                        rotated = 1;
-                        // rows, then columns, of the 2 x 2 diagonal block
-                        const T r00 = jac_comb(c, app, -s, apq), r01 = jac_comb(c, apq, -s, aqq);
-                        const T r10 = jac_comb(s, app, c, apq), r11 = jac_comb(s, apq, c, aqq);
-                        A[p * pitch + p] = jac_comb(c, r00, -s, r01);
-                        A[p * pitch + q] = jac_comb(s, r00, c, r01);
-                        A[q * pitch + q] = jac_comb(s, r10, c, r11);
-                    }
-                }
-                pp_[k] = (unsigned char)p; qq_[k] = (unsigned char)min(q, 255); cc_[k] = c; ss_[k] = s;
-                on_[k] = (unsigned char)(q < n ? on : 2);      // 2: the pair of the padding index
-            }
-            __syncthreads();
+            const unsigned char *pp_ = pp2[r & 1], *qq_ = qq2[r & 1], *on_ = on2[r & 1];
+            const T* cc_ = reinterpret_cast<const T*>(cc_raw) + (r & 1) * kJacMaxHalf;
+            const T* ss_ = reinterpret_cast<const T*>(ss_raw) + (r & 1) * kJacMaxHalf;
             // the other 2 x 2 blocks (pair l > pair k), t = l (l - 1) / 2 + k
             for (int t = threadIdx.x; t < nblk; t += blockDim.x) {
                 int l = (int)((1.0f + sqrtf(8.0f * (float)t + 1.0f)) * 0.5f);
@@ -510,16 +523,34 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
                 if (ol != 2) *e1 = x1;
                 *e0 = x0;
             }
-            // rows p, q of V^T (a warp per pair)
-            for (int k = warp; k < half; k += nwarp) {
-                if (on_[k] != 1) continue;
-                T* const vp = Vt + pp_[k] * n;
-                T* const vq = Vt + qq_[k] * n;
-                const T c = cc_[k], s = ss_[k], ns = -s;
-                for (int i = lane; i < n; i += 32) {
-                    const T vx = vp[i], vy = vq[i];
-                    vp[i] = jac_comb(c, vx, ns, vy);
-                    vq[i] = jac_comb(s, vx, c, vy);
+            __syncthreads();
+            // the next round's rotations, and beside them rows p, q of V^T
+            if (r + 1 < rounds) rotations(r + 1);
+            if (vthread >= 0) {
+                int k = vthread / n, i = vthread % n;
+                while (k < half) {
+                    T x[4], y[4];
+                    T* at[4];
+                    int kk[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        kk[u] = k < half && on_[k] == 1 ? k : -1;
+                        if (kk[u] >= 0) {
+                            at[u] = Vt + pp_[k] * n + i;
+                            x[u] = *at[u];
+                            y[u] = at[u][(qq_[k] - pp_[k]) * n];
+                        }
+                        k += vdk;
+                        i += vdi;
+                        if (i >= n) { i -= n; ++k; }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (kk[u] >= 0) {
+                            const T c = cc_[kk[u]], s = ss_[kk[u]];
+                            *at[u] = jac_comb(c, x[u], -s, y[u]);
+                            at[u][(qq_[kk[u]] - pp_[kk[u]]) * n] = jac_comb(s, x[u], c, y[u]);
+                        }
                 }
             }
             __syncthreads();
