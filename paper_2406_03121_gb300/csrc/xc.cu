@@ -29,6 +29,7 @@ constexpr int kNTheta = 16, kNPhi = 32;
 constexpr int kFuncThreads = 128;                   // points per block of the functional
 constexpr int kVxcThreads = 256, kVxcTile = 64;     // threads and function tile of the V_xc reduction
 constexpr int kVxcMaxEl = kVxcTile * kVxcTile / kVxcThreads;   // elements per thread at most
+constexpr int kLogBins = 128;                       // entries of the logarithm table
 constexpr double kRhoMin = 1e-14;   // points with less density carry no exchange-correlation energy
 
 double radius_of(int Z)
@@ -68,10 +69,10 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w)
 }
 
 // ------------------------------------------------------------------------------------------ kernels
-// Points and weights before the partition, one thread per point.  tab: the angular table (cos theta,
-// sin theta, weight for kNTheta; cos phi, sin phi for kNPhi), then per radial grid its radii and weights.
+// Points and weights before the partition, one thread per point.  tab (after the table of log_1p): the
+// angular table (cos theta, sin theta, weight for kNTheta; cos phi, sin phi for kNPhi), then per radial grid its radii and weights.
 // (Tabulated on the host and copied, the 3.3 million points of 64 H2 took about 70 ms of a call; here 0.05.)
-constexpr int kAngular = kNTheta * kNPhi, kAngularTab = 3 * kNTheta + 2 * kNPhi;
+constexpr int kAngular = kNTheta * kNPhi, kAngularAt = 2 * kLogBins, kAngularTab = kAngularAt + 3 * kNTheta + 2 * kNPhi;
 constexpr int kRadialMax = 75, kGridThreads = 256, kBlocksPerAtom = kRadialMax * kAngular / kGridThreads;
 static_assert(kRadialMax * kAngular % kGridThreads == 0, "whole blocks per atom");
 
@@ -85,12 +86,13 @@ __global__ void __launch_bounds__(kGridThreads) k_grid(const double* __restrict_
     const int i = t / kAngular, th = t % kAngular / kNPhi, ph = t % kNPhi, nr = radial_n[A];
     if (i >= nr) return;
     const double* rad = tab + radial_at[A];
-    const double r = rad[i], st = tab[kNTheta + th];
+    const double* ang = tab + kAngularAt;
+    const double r = rad[i], st = ang[kNTheta + th];
     const long long p = abase[A] + t;
-    pts[3 * p] = xyz[3 * A] + r * st * tab[3 * kNTheta + ph];
-    pts[3 * p + 1] = xyz[3 * A + 1] + r * st * tab[3 * kNTheta + kNPhi + ph];
-    pts[3 * p + 2] = xyz[3 * A + 2] + r * tab[th];
-    w[p] = rad[nr + i] * tab[2 * kNTheta + th] * 2.0 * M_PI / kNPhi;
+    pts[3 * p] = xyz[3 * A] + r * st * ang[3 * kNTheta + ph];
+    pts[3 * p + 1] = xyz[3 * A + 1] + r * st * ang[3 * kNTheta + kNPhi + ph];
+    pts[3 * p + 2] = xyz[3 * A + 2] + r * ang[th];
+    w[p] = rad[nr + i] * ang[2 * kNTheta + th] * 2.0 * M_PI / kNPhi;
     atom[p] = A;
 }
 
@@ -202,16 +204,66 @@ __global__ void k_ao(AoArgs a)
     }
 }
 
+// Roots, reciprocals and logarithms of the functional in few FP64 instructions (each takes 16 cycles of an
+// SM; the library's log1p, rcbrt, sqrt and division took most of an LDA point's): an FP32
+// estimate, relative error e below 1e-5, and the first terms of the series in e, whose next is below 1e-17.
+// x^(-1/3) for 1e-14 <= x (an FP32 number): (1 - e)^(-1/3) = 1 + e/3 + 2/9 e^2, e = 1 - x y^3
+__device__ __forceinline__ double inv_cbrt(double x)
+{
+    if (x > 1e30) return rcbrt(x);
+    const double y = f2d_alu(exp2f(log2f(d2f_alu(x)) * (-1.0f / 3.0f)));
+    const double e = fma(-x, y * y * y, 1.0);
+    return fma(y * e, fma(e, 2.0 / 9.0, 1.0 / 3.0), y);
+}
+// x^(1/2) = x x^(-1/2), (1 - e)^(-1/2) = 1 + e/2 + 3/8 e^2, e = 1 - x y^2
+__device__ __forceinline__ double fast_sqrt(double x)
+{
+    const float f = d2f_alu(x);
+    if (f < 1e-30f) return sqrt(x);
+    const double y = f2d_alu(rsqrtf(f));
+    const double e = fma(-x * y, y, 1.0);
+    return x * fma(y * e, fma(e, 0.375, 0.5), y);
+}
+// 1 / x: (1 - e)^(-1) = 1 + e + e^2, e = 1 - x y
+__device__ __forceinline__ double fast_inv(double x)
+{
+    const float f = d2f_alu(x);
+    if (f < 1e-30f) return 1.0 / x;
+    const double y = f2d_alu(__frcp_rn(f));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// log(1 + y), y >= 0: 1 + y = 2^k m, m c = 1 + w with c about 1/m from a table of 128 (c, -log c) over the
+// leading bits of m (c = 1 in the first, so that small y keep their relative accuracy), and the series of
+// log(1 + w) to w^8 (|w| <= 1/128).  What 1 + y rounds off goes into w.
+__device__ __forceinline__ double log_1p(double y, const double2* __restrict__ tab)
+{
+    const double z = 1.0 + y, lost = y - (z - 1.0);
+    const int hi = __double2hiint(z), k = (hi >> 20) - 1023;
+    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(z));
+    const double2 t = __ldg(tab + ((hi >> 13) & (kLogBins - 1)));
+    const double w = fma(lost * __hiloint2double((1023 - k) << 20, 0), t.x, fma(m, t.x, -1.0));
+    double p = 1.0 / 7 - w * (1.0 / 8);
+    p = -1.0 / 6 + w * p;
+    p = 1.0 / 5 + w * p;
+    p = -1.0 / 4 + w * p;
+    p = 1.0 / 3 + w * p;
+    p = -1.0 / 2 + w * p;
+    p = w + w * w * p;
+    const double kd = __hiloint2double(0x43300000, k ^ (int)0x80000000) - 4503601774854144.0;   // k without I2F
+    return y < 1e300 ? fma(kd, M_LN2, t.y + p) : log1p(y);
+}
+
 // Perdew-Wang 1992 correlation energy per electron (closed shell) and its derivative in rs, from rs
 // and 1 / rs.  One division: log(1 + 1/Q) and dQ / (Q (Q + 1)) share 1 / (Q (Q + 1)).
-__device__ __forceinline__ void pw92(double rs, double irs, double& ec, double& dec)
+__device__ __forceinline__ void pw92(double rs, double irs, const double2* __restrict__ logs, double& ec, double& dec)
 {
     const double A = 0.031091, a1 = 0.21370, b1 = 7.5957, b2 = 3.5876, b3 = 1.6382, b4 = 0.49294;
-    const double srs = sqrt(rs);
+    const double srs = fast_sqrt(rs);
     const double Q = 2.0 * A * srs * (b1 + srs * (b2 + srs * (b3 + srs * b4)));
     const double dQ = 2.0 * A * (0.5 * b1 * srs * irs + b2 + 1.5 * b3 * srs + 2.0 * b4 * rs);
-    const double r = 1.0 / (Q * (Q + 1.0));
-    const double L = log1p((Q + 1.0) * r);
+    const double r = fast_inv(Q * (Q + 1.0));
+    const double L = log_1p((Q + 1.0) * r, logs);
     ec = -2.0 * A * (1.0 + a1 * rs) * L;
     dec = -2.0 * A * a1 * L + 2.0 * A * (1.0 + a1 * rs) * dQ * r;
 }
@@ -227,17 +279,18 @@ struct FuncArgs {
     const double* w;
     double* vrho;            // [npts] w * d e / d rho
     double* vgrad;           // [npts][3] w * 2 d e / d sigma * grad rho (PBE)
+    const double2* logs;     // table of log_1p
     double* Exc;             // [nmol] accumulated
 };
 
 // density, its gradient, and the functional at every point of a molecule (grid.y = molecule, one
 // thread per point); E_xc accumulated per molecule.
-// Bound: the FP64 pipe (two FMA lanes per SM and clock): n^2 FMAs per point for D phi and about 100
-// (LDA) to 200 (PBE) instructions of the functional.  So the memory side only has to stay out of the
+// Bound: the FP64 pipe (two FMA lanes per SM and clock): n^2 FMAs per point for D phi and about 80
+// (LDA) to 170 (PBE) instructions of the functional.  So the memory side only has to stay out of the
 // way: phi function by function (coalesced, re-read from L1), D as warp-uniform loads, four rows of D
 // per pass so that four accumulation chains hide the FMA latency.  The functional works from
-// rho^(-1/3) and multiplies where it can: one division for LDA, four for PBE.  CH4 / 6-31G / PBE (17
-// functions, 140,800 points): 231 -> 167 us; 64 H2 (51,200 points each), LDA: 729 -> 546 us.
+// rho^(-1/3) and multiplies where it can.  CH4 / 6-31G / PBE (17 functions, 140,800 points): 231 -> 155 us
+// (167 with the library's roots and logarithms); 64 H2 (51,200 points each), LDA: 729 -> 445 us (546).
 template <int KIND>
 __global__ void __launch_bounds__(kFuncThreads) k_functional(FuncArgs f)
 {
@@ -285,14 +338,14 @@ __global__ void __launch_bounds__(kFuncThreads) k_functional(FuncArgs f)
         }
         double vr = 0.0, vs = 0.0;
         if (rho > kRhoMin) {
-            const double ic = rcbrt(rho), c13 = rho * ic * ic;    // rho^(-1/3), rho^(1/3)
+            const double ic = inv_cbrt(rho), c13 = rho * ic * ic;    // rho^(-1/3), rho^(1/3)
             const double cx = 0.7385587663820224;    // (3/4)(3/pi)^(1/3)
             const double ex = -cx * rho * c13;
             const double vx = -(4.0 / 3.0) * cx * c13;
             const double k_rs = 0.6203504908994001;       // (3/(4 pi))^(1/3)
             const double rs = k_rs * ic;
             double ec, dec;
-            pw92(rs, c13 * (1.0 / k_rs), ec, dec);
+            pw92(rs, c13 * (1.0 / k_rs), f.logs, ec, dec);
             const double rdec = -(1.0 / 3.0) * dec * rs;   // rho d ec / d rho
             if (KIND == 1) {
                 e = ex + rho * ec;
@@ -323,7 +376,7 @@ __global__ void __launch_bounds__(kFuncThreads) k_functional(FuncArgs f)
                 const double M = 1.0 + au + au * au;
                 const double N = bg * u * (1.0 + au);
                 const double rMN = 1.0 / (M * (M + N));        // dH/dy / M^2 = gamma rMN
-                const double H = gamma * log1p(N * (M + N) * rMN);
+                const double H = gamma * log_1p(N * (M + N) * rMN, f.logs);
                 const double dH_du = gamma * rMN * bg * (1.0 + 2.0 * au);
                 const double dH_dA = -gamma * rMN * bg * u * u * u * A * (2.0 + au);
                 e = ex * F + rho * (ec + H);
@@ -493,19 +546,25 @@ mess_status mess_xc_prepare(mess_basis* b, cudaStream_t s)
 {
     XcState& X = b->xc;
     if (X.ready) return MESS_OK;
-    // angular table, then the radial grid of every element present
+    // table of log_1p, angular table, then the radial grid of every element present
     std::vector<double> tab((size_t)kAngularTab);
+    for (int i = 0; i < kLogBins; ++i) {
+        const double c = i ? 1.0 / (1.0 + (i + 0.5) / kLogBins) : 1.0;
+        tab[2 * i] = c;
+        tab[2 * i + 1] = -log(c);
+    }
     {
         std::vector<double> ct, wt;
         gauss_legendre(kNTheta, ct, wt);
+        double* ang = tab.data() + kAngularAt;
         for (int t = 0; t < kNTheta; ++t) {
-            tab[t] = ct[t];
-            tab[kNTheta + t] = sqrt(1.0 - ct[t] * ct[t]);
-            tab[2 * kNTheta + t] = wt[t];
+            ang[t] = ct[t];
+            ang[kNTheta + t] = sqrt(1.0 - ct[t] * ct[t]);
+            ang[2 * kNTheta + t] = wt[t];
         }
         for (int k = 0; k < kNPhi; ++k) {
-            tab[3 * kNTheta + k] = cos(2.0 * M_PI * k / kNPhi);
-            tab[3 * kNTheta + kNPhi + k] = sin(2.0 * M_PI * k / kNPhi);
+            ang[3 * kNTheta + k] = cos(2.0 * M_PI * k / kNPhi);
+            ang[3 * kNTheta + kNPhi + k] = sin(2.0 * M_PI * k / kNPhi);
         }
     }
     std::vector<int> at_of_z(128, -1), radial_at(b->natom), radial_n(b->natom), atom_mol(b->natom);
@@ -590,7 +649,8 @@ mess_status mess_xc_eval(mess_basis* b, int kind, const double* dD, double* dV, 
     MESS_CUDA_TRY(cudaMemsetAsync(dExc, 0, sizeof(double) * b->nmol, s));
     MESS_CUDA_TRY(cudaMemsetAsync(dV, 0, sizeof(double) * b->packed, s));
     if (X.npts == 0) return MESS_OK;
-    FuncArgs f{X.phi.p, X.dphi.p, dD, b->d_mol_base.p, X.pbase.p, X.aobase.p, b->d_mol_n.p, X.w.p, X.vrho.p, X.vgrad.p, dExc};
+    FuncArgs f{X.phi.p, X.dphi.p, dD, b->d_mol_base.p, X.pbase.p, X.aobase.p, b->d_mol_n.p, X.w.p, X.vrho.p, X.vgrad.p,
+               reinterpret_cast<const double2*>(X.tab.p), dExc};
     const dim3 fgrid((unsigned)((X.mol_npts_max + kFuncThreads - 1) / kFuncThreads), (unsigned)b->nmol);
     if (kind == 2) k_functional<2><<<fgrid, kFuncThreads, 0, s>>>(f);
     else k_functional<1><<<fgrid, kFuncThreads, 0, s>>>(f);
