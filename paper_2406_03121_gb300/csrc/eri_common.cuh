@@ -475,19 +475,22 @@ __device__ __forceinline__ void jk_add(double* __restrict__ M, size_t idx, R v, 
 // contiguous ket range [kbeg[i], kbeg[i] + offs[i+1] - offs[i]) of the ket list.  A flat quartet
 // index q maps to (i, j) by a binary search over offs.
 // ------------------------------------------------------------------------------------------
-// bra of flat quartet q: the largest i with offs[i] <= q, searched between the bras of quartets
-// 32 floor(q / 32) and 32 (floor(q / 32) + 1) (a few steps instead of a search over all bras)
-__device__ __forceinline__ int find_bra(const BinLaunch& b, long long q)
+// the largest i < n with offs[i] <= q, searched between the entries of seg for q / 32 and q / 32 + 1 (a
+// few steps instead of a search over all)
+__device__ __forceinline__ int find_segment(const int* __restrict__ seg, const long long* __restrict__ offs, int n,
+                                            long long total, long long q)
 {
     const long long k = q >> 5;
-    int lo = __ldg(b.seg + k);
-    int hi = ((k + 1) << 5) < b.total ? __ldg(b.seg + k + 1) : b.nbra - 1;
+    int lo = __ldg(seg + k);
+    int hi = ((k + 1) << 5) < total ? __ldg(seg + k + 1) : n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(b.offs + mid) <= q) lo = mid; else hi = mid - 1;
+        if (__ldg(offs + mid) <= q) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
+// bra of flat quartet q
+__device__ __forceinline__ int find_bra(const BinLaunch& b, long long q) { return find_segment(b.seg, b.offs, b.nbra, b.total, q); }
 
 __device__ __forceinline__ bool warp_uniform_int(int v)
 {
@@ -644,6 +647,110 @@ constexpr int group_pitch(int nacc, int nint) { return (nacc > nint ? nacc : nin
                         G[((d * nn + c) * nn + bb) * nn + a] = v;                                   \
                     }                                                                               \
     }
+
+// hi + lo += v (error-free sum of the leading parts)
+__device__ __forceinline__ void sum_exact(df32& acc, float v)
+{
+    const df32 t = df_two_sum(acc.hi, v);
+    acc.hi = t.hi;
+    acc.lo += t.lo;
+}
+__device__ __forceinline__ void flush_exact(double* __restrict__ M, size_t idx, df32 v)
+{
+    if (v.hi != 0.f || v.lo != 0.f) atomicAdd(M + idx, f2d_alu(v.hi) + f2d_alu(v.lo));
+}
+
+// FP32 J/K kernel of one class over bra runs: one thread takes a ket cd through up to MESS_RUN_MAX bras
+// ab, ab', ... with the same first shell a.  J_cd, K_ac and K_ad then go to memory once per run instead of
+// once per quartet (summed exactly in hi + lo FP32 pairs), D_cd, D_ac and D_ad are loaded once, and so is
+// the ket.  Per quartet there remain K_bc, K_bd and the warp's sum for J_ab.  The one-thread-per-quartet
+// kernels are bound by exactly that traffic (FP64 reductions at 110 to 140 G sectors/s, 60 to 70 % of the
+// L1 and L2 throughput).  (H2O)_32 / 6-31G*, launches one at a time: (ps|ss) 2.70 -> 1.36 ms,
+// (ds|ps) 1.78 -> 0.75, (ds|ss) 1.45 -> 0.69, (ps|ps) 1.36 -> 0.61, all J/K kernels 21.6 -> 16.7.
+#define MESS_DEFINE_RUN_KERNEL(TAG, NA, NB, NC, ND)                                                 \
+    __global__ void __launch_bounds__(MESS_THREADS)                                                 \
+    k_jk_run_##TAG(const BinLaunch b, const RunLaunch r, const PairTable<float> P, const float* __restrict__ D, \
+                   double* __restrict__ J, double* __restrict__ K)                                  \
+    {                                                                                               \
+        const long long q0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;                     \
+        const bool valid = q0 < r.total;                                                            \
+        const long long q = valid ? q0 : r.total - 1;                                               \
+        const int i = find_segment(r.seg, r.offs, r.nrun, r.total, q);                              \
+        const int4 run = __ldg(r.run + i);                                                          \
+        const int j = run.z + (int)(q - __ldg(r.offs + i));                                         \
+        const KetRec* kr = b.ketrec + j;                                                            \
+        const int4 kh = ket_hdr(kr);                                                                \
+        const int kp = ket_pair(kr);                                                                \
+        const int bp0 = __ldg(b.bra + run.x);                                                       \
+        const bool live = valid && P.live(bp0);                                                     \
+        if (__all_sync(0xffffffffu, !live)) return;                                                 \
+        const KetView<float> kv = ket_view(P, bp0, kr, kh);   /* (A is the run's) */                \
+        const int m_ = __ldg(P.mol + bp0);                                                          \
+        const long long o_ = __ldg(P.mbase + m_);                                                   \
+        RunCtx<NA, NC, ND> c;                                                                       \
+        c.D = D + o_; c.J = J + o_; c.K = K + o_; c.n = __ldg(P.mn + m_);                           \
+        c.fa = __ldg(P.fa + bp0); c.fc = kh.z & 0xffff; c.fd = kh.z >> 16;                          \
+        c.uniform = warp_uniform_int(i);                                                            \
+        c.load();                                                                                   \
+        const int nb = c.uniform ? run.y : __reduce_max_sync(0xffffffffu, run.y);                   \
+        _Pragma("unroll 1") for (int t = 0; t < nb; ++t) {                                          \
+            const int bi = run.x + min(t, run.y - 1);                                               \
+            const int k0 = __ldg(b.kbeg + bi), bp = __ldg(b.bra + bi);                              \
+            const int k1 = k0 + (int)(__ldg(b.offs + bi + 1) - __ldg(b.offs + bi));                 \
+            const bool act = live && t < run.y && j >= k0 && j < k1 && P.dens_ok(bp, kp);           \
+            if (!__any_sync(0xffffffffu, act)) continue;                                            \
+            float I[(NA) * (NB) * (NC) * (ND)];                                                     \
+            eri_##TAG<float, 2, 1>(P, bp, kv, 0, I, act);                                           \
+            float s = act ? 1.0f : 0.0f;                                                            \
+            if (__ldg(P.same + bp)) s *= 0.5f;                                                      \
+            if (kh.w & 1) s *= 0.5f;                                                                \
+            if (bp == kp) s *= 0.5f;                                                                \
+            digest_run_##TAG(I, c, s, __ldg(P.fb + bp));                                            \
+        }                                                                                           \
+        c.flush();                                                                                  \
+    }
+
+// what a thread of a run keeps: the density blocks and sums that do not depend on b
+template <int NA, int NC, int ND> struct RunCtx {
+    const float* __restrict__ D;
+    double* __restrict__ J;
+    double* __restrict__ K;
+    int n, fa, fc, fd;
+    bool uniform;            // every lane of the warp is in the same run: reduce J_ab across the warp
+    float Dcd[NC * ND], Dac[NA * NC], Dad[NA * ND];
+    df32 Jcd[NC * ND], Kac[NA * NC], Kad[NA * ND];
+
+    __device__ __forceinline__ void load()
+    {
+        block<NC, ND>(Dcd, Jcd, fc, fd);
+        block<NA, NC>(Dac, Kac, fa, fc);
+        block<NA, ND>(Dad, Kad, fa, fd);
+    }
+    __device__ __forceinline__ void flush() const
+    {
+        store<NC, ND>(J, Jcd, fc, fd);
+        store<NA, NC>(K, Kac, fa, fc);
+        store<NA, ND>(K, Kad, fa, fd);
+    }
+private:
+    template <int M, int N> __device__ __forceinline__ void block(float* d, df32* sum, int r0, int c0)
+    {
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                d[i * N + j] = ldD(D + (size_t)(r0 + i) * n + c0 + j);
+                sum[i * N + j] = df32(0.f, 0.f);
+            }
+    }
+    template <int M, int N> __device__ __forceinline__ void store(double* X, const df32* sum, int r0, int c0) const
+    {
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+#pragma unroll
+            for (int j = 0; j < N; ++j) flush_exact(X, (size_t)(r0 + i) * n + c0 + j, sum[i * N + j]);
+    }
+};
 
 // Schwarz factors Q_ab = sqrt(max_{m in a, n in b} |(mn|mn)|) for a list of pairs of one class, G lanes
 // per pair: the primitive quartets of a diagonal quartet number the square of the pair's primitive

@@ -19,6 +19,7 @@ struct ClassLaunchArgs {
     int G;                       // JK: lanes per shell quartet (1, 4 or 8)
     int team;                    // JK: 1 = one warp per shell quartet (level-scheduled program)
     BinLaunch bin;               // JK / STORE
+    const RunLaunch* runs;       // JK: the FP32 one-thread kernel goes by bra runs (null: by quartets)
     const int* pairs;            // SCHWARZ: pair ids of one diagonal class
     int npairs;
     const PairTable<double>* P64_ptr;

@@ -811,6 +811,42 @@ def team_capable(info):
     return info["nvrr"] >= 40
 
 
+def run_capable(info):
+    """classes with an FP32 kernel over bra runs (MESS_DEFINE_RUN_KERNEL): straight-line code whose blocks
+    J_cd, K_ac, K_ad of a thread still fit its registers"""
+    na, nc, nd = ncart(info["la"]), ncart(info["lc"]), ncart(info["ld"])
+    return info["mode"] == "straight" and nc * nd + na * nc + na * nd <= 27
+
+
+def emit_run_digest(cls):
+    """Digestion of one quartet of a bra run: sums for J_cd, K_ac, K_ad kept by the thread, K_bc, K_bd and
+    (summed over the warp) J_ab to memory."""
+    (la, lb), (lc, ld) = cls
+    t = tag(cls)
+    na, nb, nc, nd = ncart(la), ncart(lb), ncart(lc), ncart(ld)
+    U = "#pragma unroll"
+    I = f"I[((i * {nb} + j) * {nc} + k) * {nd} + l]"
+    idx = {"i": na, "j": nb, "k": nc, "l": nd}
+    L = [f"__device__ __forceinline__ void digest_run_{t}(const float* I, RunCtx<{na}, {nc}, {nd}>& c, float s, int fb)", "{"]
+    for nm, (r0, nr), (c0, ncol) in (("Dab", ("c.fa", na), ("fb", nb)), ("Dbc", ("fb", nb), ("c.fc", nc)),
+                                     ("Dbd", ("fb", nb), ("c.fd", nd))):
+        L += [f"    float {nm}[{nr * ncol}];", U, f"    for (int i = 0; i < {nr}; ++i)", U,
+              f"        for (int j = 0; j < {ncol}; ++j) {nm}[i * {ncol} + j] = ldD(c.D + (size_t)({r0} + i) * c.n + {c0} + j);"]
+    for o1, o2, D, out in (("i", "j", "c.Dcd", "jk_add(c.J, (size_t)(c.fa + i) * c.n + fb + j, s * t, c.uniform);"),
+                           ("k", "l", "Dab", f"sum_exact(c.Jcd[k * {nd} + l], s * t);"),
+                           ("i", "k", "Dbd", f"sum_exact(c.Kac[i * {nc} + k], s * t);"),
+                           ("i", "l", "Dbc", f"sum_exact(c.Kad[i * {nd} + l], s * t);"),
+                           ("j", "k", "c.Dad", "jk_add(c.K, (size_t)(fb + j) * c.n + c.fc + k, s * t, false);"),
+                           ("j", "l", "c.Dac", "jk_add(c.K, (size_t)(fb + j) * c.n + c.fd + l, s * t, false);")):
+        s1, s2 = [x for x in "ijkl" if x not in (o1, o2)]
+        L += [U, f"    for (int {o1} = 0; {o1} < {idx[o1]}; ++{o1})", U,
+              f"        for (int {o2} = 0; {o2} < {idx[o2]}; ++{o2}) {{", "            float t = 0.f;", U,
+              f"            for (int {s1} = 0; {s1} < {idx[s1]}; ++{s1})", U,
+              f"                for (int {s2} = 0; {s2} < {idx[s2]}; ++{s2}) t += {I} * {D}[{s1} * {idx[s2]} + {s2}];",
+              f"            {out}", "        }"]
+    return "\n".join(L + ["}"]) + "\n"
+
+
 def emit_digests(cls, info):
     """The digestion of a class as the kernels call it (digest_<class>).  Straight-line classes stage
     the density blocks in registers.  The op-program classes, and the double-float path of the
@@ -905,6 +941,8 @@ def main(outdir):
         if team_capable(info) or info["mode"] == "program":
             body += "\n" + emit_team(cls, info)
         dig = emit_digests(cls, info)
+        if run_capable(info):
+            dig += "\n" + emit_run_digest(cls)
         path = os.path.join(outdir, f"eri_class_{info['tag']}.cuh")
         text = ("// Generated by gen_eri.py: do not edit.\n#pragma once\n#include \"eri_common.cuh\"\n\n"
                 + body + "\n" + dig)
@@ -924,6 +962,8 @@ def main(outdir):
         team = team_capable(info) or info["mode"] == "program"
         if team:
             u.append(f"MESS_DEFINE_TEAM_KERNEL({t})")
+        if run_capable(info):
+            u.append(f"MESS_DEFINE_RUN_KERNEL({t}, {na}, {nb}, {nc}, {nd})")
         if diag:
             u.append(f"MESS_DEFINE_SCHWARZ_KERNEL({t}, {na}, {nb}, {info['nacc']})" if info["mode"] == "straight"
                      else f"MESS_DEFINE_TEAM_SCHWARZ_KERNEL({t})")
@@ -950,6 +990,14 @@ def main(outdir):
             u += ["        return cudaErrorInvalidValue;"]
         u += ["    }",
               "    if (a.bin.total <= 0) return cudaSuccess;",
+              ] + ([
+              "    if (a.kind == MESS_KIND_JK && a.runs) {",
+              "        const long long nbr = (a.runs->total + T - 1) / T;",
+              "        if (nbr > 0x7fffffffLL) return cudaErrorInvalidConfiguration;",
+              f"        k_jk_run_{t}<<<(unsigned)nbr, T, 0, a.stream>>>(a.bin, *a.runs, *a.P32_ptr, dmat<float>(a), a.J, a.K);",
+              "        return cudaGetLastError();",
+              "    }",
+              ] if run_capable(info) else []) + [
               "    const int T1 = a.kind == MESS_KIND_JK ? jk_block_threads(a.bin.total) : T;",
               "    const long long nblk = (a.bin.total + T1 - 1) / T1;",
               "    if (nblk > 0x7fffffffLL) return cudaErrorInvalidConfiguration;",
@@ -1048,8 +1096,8 @@ def main(outdir):
            f"#define MESS_NUM_QCLASS {len(QUARTET_CLASSES)}", "",
            "// straight: kernels with G = 1, 4, 8, 32 lanes per quartet (else G = 1 only); team: a",
            "// warp-per-quartet kernel exists; line: the one-thread kernel is straight-line code (else the op",
-           "// program) in FP32 (1), FP64 (2), double-float (4)",
-           "typedef struct { int la, lb, lc, ld, L, nint, nacc, nvrr; long vrr_flops, hrr_flops; int straight, team, line; }",
+           "// program) in FP32 (1), FP64 (2), double-float (4); run: an FP32 kernel over bra runs exists",
+           "typedef struct { int la, lb, lc, ld, L, nint, nacc, nvrr; long vrr_flops, hrr_flops; int straight, team, line, run; }",
            "    mess_qclass_info;",
            "static const mess_qclass_info MESS_QCLASS[MESS_NUM_QCLASS] = {"]
     for f in infos:
@@ -1057,7 +1105,7 @@ def main(outdir):
         tm = 1 if (team_capable(f) or f["mode"] == "program") else 0
         ln = sum({"float": 1, "double": 2, "df32": 4}[x] for x in line_types(f))
         tab.append(f"    {{{f['la']}, {f['lb']}, {f['lc']}, {f['ld']}, {f['L']}, {f['nint']}, {f['nacc']}, "
-                   f"{f['nvrr']}, {f['vrr_flops']}, {f['hrr_flops']}, {st}, {tm}, {ln}}},")
+                   f"{f['nvrr']}, {f['vrr_flops']}, {f['hrr_flops']}, {st}, {tm}, {ln}, {int(run_capable(f))}}},")
     tab.append("};")
     text = "\n".join(tab) + "\n"
     path = os.path.join(outdir, "eri_classes.h")

@@ -198,7 +198,7 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
     // within one pair class); each builds its parts (FP64-class / reduced-precision split) into its
     // own arrays.  Tasks are independent and run on host threads; the parts are concatenated in task
     // order, so the bins do not depend on the threading.
-    struct Task { int p1, p2, L1, L2; std::vector<BinPart> parts; std::vector<int> bra, kbeg; std::vector<long long> offs; };
+    struct Task { int p1, p2, L1, L2; std::vector<BinPart> parts; std::vector<int> bra, kbeg; std::vector<long long> offs; std::vector<int4> run; };
     std::vector<Task> tasks;
     for (int p1 = 0; p1 < MESS_NUM_PCLASS; ++p1)
         for (int p2 = 0; p2 <= p1; ++p2)
@@ -208,7 +208,7 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
                     if ((p1 == p2 && h2 > h1) || (x1 && x2)) continue;
                     const int L1 = MESS_LIST(x1, p1, h1 % MESS_NGROUP), L2 = MESS_LIST(x2, p2, h2 % MESS_NGROUP);
                     if (b->class_list[L1].empty() || b->class_list[L2].empty()) continue;
-                    tasks.push_back(Task{p1, p2, L1, L2, {}, {}, {}, {}});
+                    tasks.push_back(Task{p1, p2, L1, L2, {}, {}, {}, {}, {}});
                 }
     auto run_task = [&](Task& T) {
         const int p1 = T.p1, p2 = T.p2, L1 = T.L1, L2 = T.L2;
@@ -272,6 +272,43 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
             }
             bp.nbra = (int)bra.size() - bp.bra_off;
             offs.push_back(bp.total);
+            if (!fp64 && MESS_QCLASS[bp.qclass].run && bp.total >= MESS_RUN_MIN && bp.prim_quartets <= MESS_RUN_PRIM * bp.total) {
+                // the bras of one first shell together, then runs of them, their kets the union of the bras'
+                std::vector<int> order(bp.nbra);
+                std::iota(order.begin(), order.end(), 0);
+                const std::vector<int> bra0(bra.begin() + bp.bra_off, bra.end()), kbeg0(kbeg.begin() + bp.bra_off, kbeg.end());
+                const std::vector<long long> offs0(offs.begin() + bp.offs_off, offs.end());
+                std::stable_sort(order.begin(), order.end(),
+                                 [&](int x, int y) { return b->pair_a[bra0[x]] < b->pair_a[bra0[y]]; });
+                long long at = 0;
+                for (int i = 0; i < bp.nbra; ++i) {
+                    const int x = order[i];
+                    bra[bp.bra_off + i] = bra0[x];
+                    kbeg[bp.bra_off + i] = kbeg0[x];
+                    offs[bp.offs_off + i] = at;
+                    at += offs0[x + 1] - offs0[x];
+                }
+                bp.run_off = T.run.size();
+                bp.run_offs_off = offs.size();
+                const long long* po = offs.data() + bp.offs_off;
+                std::vector<long long> roffs;
+                for (int i = 0; i < bp.nbra;) {
+                    const int a = b->pair_a[bra[bp.bra_off + i]];
+                    int n = 0, k0 = INT32_MAX, k1 = 0;
+                    for (; n < MESS_RUN_MAX && i + n < bp.nbra && b->pair_a[bra[bp.bra_off + i + n]] == a; ++n) {
+                        const int beg = kbeg[bp.bra_off + i + n];
+                        k0 = std::min(k0, beg);
+                        k1 = std::max(k1, beg + (int)(po[i + n + 1] - po[i + n]));
+                    }
+                    T.run.push_back(make_int4(i, n, k0, 0));
+                    roffs.push_back(bp.run_total);
+                    bp.run_total += k1 - k0;
+                    i += n;
+                }
+                bp.nrun = (int)roffs.size();
+                roffs.push_back(bp.run_total);
+                offs.insert(offs.end(), roffs.begin(), roffs.end());
+            }
             if (bp.nbra > 0) T.parts.push_back(bp);
             else offs.resize(bp.offs_off);
         }
@@ -290,30 +327,38 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
     }
     std::vector<int> bra, kbeg;
     std::vector<long long> offs;
+    std::vector<int4> run;
     for (Task& T : tasks) {
         for (BinPart bp : T.parts) {
             bp.bra_off += (int)bra.size();
             bp.offs_off += offs.size();
+            bp.run_offs_off += offs.size();
+            bp.run_off += run.size();
             B.parts.push_back(bp);
         }
+        run.insert(run.end(), T.run.begin(), T.run.end());
         bra.insert(bra.end(), T.bra.begin(), T.bra.end());
         kbeg.insert(kbeg.end(), T.kbeg.begin(), T.kbeg.end());
         offs.insert(offs.end(), T.offs.begin(), T.offs.end());
     }
     tasks.clear();
-    // per part, the bra of every 32nd quartet
+    // per part, the bra of every 32nd quartet (and the run of every 32nd thread)
     std::vector<int> seg;
-    for (BinPart& p : B.parts) {
-        p.seg_off = seg.size();
-        const long long* po = offs.data() + p.offs_off;   // [nbra + 1]
+    auto add_seg = [&](const long long* po, int n, long long total) {
+        const size_t at = seg.size();
         int i = 0;
-        for (long long q = 0; q < p.total; q += 32) {
-            while (i + 1 < p.nbra && po[i + 1] <= q) ++i;
+        for (long long q = 0; q < total; q += 32) {
+            while (i + 1 < n && po[i + 1] <= q) ++i;
             seg.push_back(i);
         }
+        return at;
+    };
+    for (BinPart& p : B.parts) {
+        p.seg_off = add_seg(offs.data() + p.offs_off, p.nbra, p.total);
+        if (p.nrun) p.run_seg_off = add_seg(offs.data() + p.run_offs_off, p.nrun, p.run_total);
     }
     if (B.bra.upload(bra) != cudaSuccess || B.kbeg.upload(kbeg) != cudaSuccess || B.offs.upload(offs) != cudaSuccess ||
-        B.seg.upload(seg) != cudaSuccess) {
+        B.seg.upload(seg) != cudaSuccess || B.run.upload(run) != cudaSuccess) {
         mess_set_error("uploading quartet bins failed");
         B.tau = -1.0;
         return MESS_ECUDA;
@@ -396,6 +441,14 @@ static BinLaunch bin_launch(const mess_basis* b, const BinPart& p)
     L.total = p.total;
     return L;
 }
+
+static RunLaunch run_launch(const mess_basis* b, const BinPart& p)
+{
+    return RunLaunch{b->bins.run.p + p.run_off, b->bins.offs.p + p.run_offs_off, b->bins.seg.p + p.run_seg_off, p.nrun,
+                     p.run_total};
+}
+// whether the launch of a part in this shape goes by bra runs
+static bool by_runs(const BinPart& p, int G, int team, int mode) { return p.nrun && G == 1 && !team && mode == MESS_MODE_FP32; }
 
 // ------------------------------------------------------------------------------------------ create
 // Append one molecule (atoms and already normalised shells) to a basis under construction.
@@ -785,7 +838,7 @@ void mess_free_basis(mess_basis* b)
     for (auto& d : b->d_class_list) d.free();
     for (auto& d : b->d_ketrec) d.free();
     b->d_pair_rec.free();
-    b->bins.bra.free(); b->bins.kbeg.free(); b->bins.offs.free(); b->bins.seg.free();
+    b->bins.bra.free(); b->bins.kbeg.free(); b->bins.offs.free(); b->bins.seg.free(); b->bins.run.free();
     mess_free_jk_graphs(b);
     b->d_D32.free(); b->d_Ddf.free(); b->d_stage.free();
     mess_free_xc(b);
@@ -1103,6 +1156,8 @@ static mess_status jk_enqueue(mess_basis* b, const mess_jk_opts& o, const double
         a.G = shape[k].G;
         a.team = shape[k].team;
         a.bin = bin_launch(b, p);
+        const RunLaunch runs = run_launch(b, p);
+        a.runs = by_runs(p, a.G, a.team, a.mode) ? &runs : nullptr;
         a.P64_ptr = &b->P64;
         a.P32_ptr = &b->P32;
         a.Pdf_ptr = &b->Pdf;
@@ -1436,6 +1491,8 @@ static mess_status jk_autotune_device(mess_basis* b, const double* dD, double* d
             a.G = v.G;
             a.team = v.team;
             a.bin = bin_launch(b, p);
+            const RunLaunch runs = run_launch(b, p);
+            a.runs = by_runs(p, v.G, v.team, v.mode) ? &runs : nullptr;
             a.P64_ptr = &b->P64;
             a.P32_ptr = &b->P32;
             a.Pdf_ptr = &b->Pdf;

@@ -68,3 +68,22 @@ struct BinLaunch {
     int nbra;
     long long total;
 };
+
+// A bin's bras in runs that share their first shell (FP32 parts, see k_jk_run_*): one thread per (run,
+// ket), ket ranges as the union over the run's bras.
+#define MESS_RUN_MAX 8            // bras per run at most
+// A part is laid out in runs when it has many shell quartets (a run takes an eighth of the threads) with few
+// primitive quartets each (with more, the primitives bound it, and the registers that hold the run's sums cost
+// warps).  One thread per quartet -> runs, (H2O)_32 / 6-31G* and (H2O)_64 / STO-3G, 13 M (ps|ss) quartets of 4
+// primitive quartets 1830 -> 548 us, 3.7 M (ds|ps) of 3 1487 -> 457, 3.2 M (ps|ss) of 13 354 -> 290, 1.9 M of 14
+// 182 -> 188; of 46: 12 M (ss|ss) 1555 -> 1548, 1.5 M (pp|ss) 353 -> 455, 0.7 M (pp|ps) 343 -> 485.  16 bras per
+// run instead of 8: 0 to 20 % slower.
+#define MESS_RUN_MIN (1LL << 19)
+#define MESS_RUN_PRIM 16
+struct RunLaunch {
+    const int4* run;         // [nrun] first bra, number of bras, first ket, 0
+    const long long* offs;   // [nrun + 1] exclusive prefix of the runs' ket counts
+    const int* seg;          // [ceil(total / 32)] run of thread 32 k
+    int nrun;
+    long long total;         // threads
+};

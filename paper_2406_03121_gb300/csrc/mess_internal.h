@@ -83,6 +83,9 @@ struct BinPart {
     long long prim_quartets;
     size_t offs_off;       // into offs
     size_t seg_off;        // into seg: bra index of every 32nd quartet of the part
+    int nrun = 0;          // bra runs (0: the part is not laid out in runs)
+    long long run_total = 0;                           // threads of the run kernel
+    size_t run_off = 0, run_offs_off = 0, run_seg_off = 0;   // into run, offs, seg
 };
 
 struct BinSet {
@@ -94,6 +97,7 @@ struct BinSet {
     DevBuf<int> bra, kbeg;
     DevBuf<long long> offs;
     DevBuf<int> seg;
+    DevBuf<int4> run;
 };
 
 // An instantiated CUDA graph of one J/K build: the bins' generation, the options that select
