@@ -52,16 +52,16 @@ mess_status mess_boys_device(MessBoysTables* out)
         static std::vector<double> h64;
         static std::vector<float4> h32, hdf;
         if (h64.empty()) {
-            // one table at the finest step (1/64); the others take every second and every fourth row
-            static_assert(MESS_BOYSDF_INV_DT == 2 * MESS_BOYS64_INV_DT && MESS_BOYSDF_INV_DT == 4 * MESS_BOYS32_INV_DT, "steps");
-            const int nrow = std::max({2 * MESS_BOYS64_NROW, MESS_BOYSDF_NROW, 4 * MESS_BOYS32_NROW});
+            // one table at the finest step (1/128); the others take every second and every fourth row
+            static_assert(MESS_BOYS32_INV_DT == 2 * MESS_BOYSDF_INV_DT && MESS_BOYS32_INV_DT == 4 * MESS_BOYS64_INV_DT, "steps");
+            const int nrow = std::max({4 * MESS_BOYS64_NROW, 2 * MESS_BOYSDF_NROW, MESS_BOYS32_NROW});
             std::vector<double> t;
-            mess_boys_table(t, nrow, 1.0 / MESS_BOYSDF_INV_DT);
+            mess_boys_table(t, nrow, 1.0 / MESS_BOYS32_INV_DT);
             const double fact[7] = {1.0, 1.0, 2.0, 6.0, 24.0, 120.0, 720.0};
             std::vector<float4> df((size_t)MESS_BOYS_NL * MESS_BOYSDF_NROW * 3);
             for (int L = 0; L < MESS_BOYS_NL; ++L)
                 for (int k = 0; k < MESS_BOYSDF_NROW; ++k) {
-                    const double* row = t.data() + (size_t)k * MESS_BOYS_NCOL;
+                    const double* row = t.data() + (size_t)(2 * k) * MESS_BOYS_NCOL;
                     float hi[7], lo[7];
                     for (int j = 0; j < 7; ++j) {
                         const double c = j < 6 ? row[L + j] / fact[j] : row[MESS_BOYS_NF];
@@ -76,14 +76,19 @@ mess_status mess_boys_device(MessBoysTables* out)
             std::vector<float4> f32((size_t)MESS_BOYS_NL * MESS_BOYS32_NROW);
             for (int L = 0; L < MESS_BOYS_NL; ++L)
                 for (int k = 0; k < MESS_BOYS32_NROW; ++k) {
-                    const double* row = t.data() + (size_t)(4 * k) * MESS_BOYS_NCOL;
+                    const double* row = t.data() + (size_t)k * MESS_BOYS_NCOL;
+                    if (L == 0) {
+                        constexpr int step = (int)(MESS_BOYS32_INV_DT / MESS_BOYS32_INV_DT0);
+                        if (k % step == 0) f32[k / step] = make_float4((float)row[0], (float)row[1], (float)(row[2] / 2), (float)(row[3] / 6));
+                        continue;
+                    }
                     f32[(size_t)L * MESS_BOYS32_NROW + k] =
-                        make_float4((float)row[L], (float)row[L + 1], (float)row[L + 2], (float)row[MESS_BOYS_NF]);
+                        make_float4((float)row[L], (float)row[L + 1], (float)(0.5 * row[L + 2]), (float)row[MESS_BOYS_NF]);
                 }
             std::vector<double> f64((size_t)MESS_BOYS_NL * MESS_BOYS64_NROW * 8);
             for (int L = 0; L < MESS_BOYS_NL; ++L)
                 for (int k = 0; k < MESS_BOYS64_NROW; ++k) {
-                    const double* row = t.data() + (size_t)(2 * k) * MESS_BOYS_NCOL;
+                    const double* row = t.data() + (size_t)(4 * k) * MESS_BOYS_NCOL;
                     double* o = f64.data() + ((size_t)L * MESS_BOYS64_NROW + k) * 8;
                     for (int j = 0; j < 7; ++j) o[j] = row[L + j] / fact[j];
                     o[7] = row[MESS_BOYS_NF];

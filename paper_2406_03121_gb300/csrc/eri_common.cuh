@@ -98,7 +98,7 @@ template <typename R> struct PairTable {
     const long long* __restrict__ mbase;     // [nmol] offset of the molecule's n x n block (packed matrices)
     const int* __restrict__ mn;              // [nmol] basis functions of the molecule (row stride)
     const double* __restrict__ boys64;       // FP64 Boys rows per order L (mess_device.h)
-    const float4* __restrict__ boys32v;      // FP32 rows per order L: [L][row] {F_L, F_L+1, F_L+2, exp(-T_k)}
+    const float4* __restrict__ boys32v;      // FP32 rows per order L: [L][row] {F_L, F_L+1, F_L+2 / 2, exp(-T_k)}; L = 0: F_3 / 6 last
     const float4* __restrict__ boysdf;       // double-float rows per order L
     // per molecule: 0 = left the computation (a converged molecule of a batched SCF): its quartets
     // are skipped by the J/K kernels.  Null: every molecule takes part.
@@ -258,53 +258,52 @@ template <int L> __device__ __forceinline__ void boys_large_f64(double T, double
     }
 }
 
-template <int L> __device__ __forceinline__ void boys_small_f32(float T, float* F, const float4* __restrict__ tabv)
-{
-    // nearest grid index without F2I / I2F conversions (those issue on the slow FP64 pipe): adding
-    // 1.5 * 2^23 rounds T / dT to an integer held in the low mantissa bits (0 <= T / dT < 2^22)
-    const float r = fmaf(T, (float)MESS_BOYS32_INV_DT, 12582912.0f);
-    const int k = __float_as_int(r) - 0x4B400000;
-    const float kf = r - 12582912.0f;                  // k as a float, exactly
-    const float x = kf * (float)MESS_BOYS32_DT - T;    // T_k - T (T_k exact), |x| <= 1/32
-    // One 16-byte row: F_L, F_L+1, F_L+2 and exp(-T_k), each rounded once from the FP64 grid.
-    // F_L+3 and F_L+4 at T_k for the third- and fourth-order terms (at most 5e-6 and 4e-8 of F_L,
-    // so a few correct digits suffice; the fourth is kept because dropping it would bias every FP32
-    // integral with one sign) come from the upward recursion F_m+1 = ((2m+1) F_m - exp(-T_k)) / (2 T_k),
-    // F_m(0) = 1/(2m+1) at the first grid point.
-    const float4 a = __ldg(tabv + (size_t)L * MESS_BOYS32_NROW + k);
-    const float ek = a.w;
-    float f3, f4;
-    if (k > 0) {
-        const float h = __fdividef(0.5f * (float)MESS_BOYS32_INV_DT, kf);   // 1 / (2 T_k)
-        f3 = ((float)(2 * L + 5) * a.z - ek) * h;
-        f4 = ((float)(2 * L + 7) * f3 - ek) * h;
-    } else {
-        f3 = 1.0f / (float)(2 * L + 7);
-        f4 = 1.0f / (float)(2 * L + 9);
-    }
-    float s = f4;
-    s = f3 + s * x * 0.25f;
-    s = a.z + s * x * (1.0f / 3);
-    s = a.y + s * x * 0.5f;
-    s = a.x + s * x;
-    F[L] = s;
-    if (L == 0) return;
-    // exp(-T) = exp(-T_k) exp(x), exp(x) to fourth order (|x| <= 1/32: the next term is below 2e-9)
-    const float e = ek * (1.0f + x * (1.0f + x * (0.5f + x * (1.0f / 6 + x * (1.0f / 24)))));
-    const float t2 = 2.0f * T;
-#pragma unroll
-    for (int m = L; m >= 1; --m) F[m - 1] = (t2 * F[m] + e) * (1.0f / (2 * m - 1));
-}
-
 template <int L> __device__ __forceinline__ void boys_large_f32(float T, float* F)
 {
-    const float rt = rsqrtf(T);
+    const float rt = rsqrt_ftz(T);
     F[0] = 0.886226925f * rt;
     if (L > 0) {
         const float e = __expf(-T);
         const float h = 0.5f * rt * rt;
 #pragma unroll
         for (int m = 0; m < L; ++m) F[m + 1] = ((2 * m + 1) * F[m] - e) * h;
+    }
+}
+
+// FP32.  The lanes of a warp lie on both sides of the grid's end, and the two sides of a branch would run one after
+// the other: the asymptote is formed for every lane (exp(-T) left out: 2e-16 at 36, below 1e-8 of 2 T F_8) and
+// replaced below the end.  For L <= 1 the lanes above it skip the rest, since the gather of rows fills the L1 data
+// pipe there (95 % for (ss|ss)); for the longer recursions the selection is 1 to 8 % faster.  Instructions, not
+// loads, bound those, so a row holds what order 2 at a step of 1/128 needs (three FMAs, where order 4 at 1/16
+// took the upward recursion for two of its terms and a division).
+// Batch of 256 alkanes / STO-3G, per three builds: (ps|ss) 15.9 -> 12.6 ms, (ps|ps) 6.7 -> 5.8, (pp|ss) 3.3 -> 2.6,
+// (ss|ss) 10.8 -> 10.3; (H2O)_32 / 6-31G*, (ss|ss) 894 -> 733 us, (ps|ss) 1349 -> 1253.
+template <int L> __device__ __forceinline__ void boys_f32(float T, float* F, const float4* __restrict__ tabv)
+{
+    const bool far = !(T < (float)MESS_BOYS_TMAX32);
+    const float rt = rsqrt_ftz(T), h = 0.5f * rt * rt;
+    F[0] = 0.886226925f * rt;   // sqrt(pi)/2 / sqrt(T)
+#pragma unroll
+    for (int m = 0; m < L; ++m) F[m + 1] = F[m] * ((float)(2 * m + 1) * h);
+    if (L <= 1 && far) return;
+    const float Tc = fminf(T, (float)MESS_BOYS_TMAX32);
+    // nearest grid index without F2I / I2F conversions (those issue on the slow FP64 pipe): adding
+    // 1.5 * 2^23 rounds T / dT to an integer held in the low mantissa bits (0 <= T / dT < 2^22)
+    constexpr float inv_dt = L > 0 ? (float)MESS_BOYS32_INV_DT : (float)MESS_BOYS32_INV_DT0;
+    const float r = fmaf(Tc, inv_dt, 12582912.0f);
+    const int k = __float_as_int(r) - 0x4B400000;
+    const float x = fmaf(r - 12582912.0f, 1.0f / inv_dt, -Tc);    // T_k - T (exact)
+    const float4 a = __ldg(tabv + (size_t)L * MESS_BOYS32_NROW + k);
+    float d = fmaf(x, fmaf(x, L > 0 ? a.z : fmaf(x, a.w, a.z), a.y), a.x);
+    F[L] = far ? F[L] : d;
+    if (L == 0) return;
+    // exp(-T) = exp(-T_k) exp(x), exp(x) to third order (the next term is below 1e-11)
+    const float e = a.w * fmaf(x, fmaf(x, fmaf(x, 1.0f / 6, 0.5f), 1.0f), 1.0f);
+    const float t2 = 2.0f * T;
+#pragma unroll
+    for (int m = L; m >= 1; --m) {
+        d = m == 1 ? fmaf(t2, d, e) : fmaf(t2, d, e) * (1.0f / (2 * m - 1));
+        F[m - 1] = far ? F[m - 1] : d;
     }
 }
 
@@ -380,7 +379,7 @@ template <int L> struct BoysEval<float, L, 1> {
 template <int L> struct BoysEval<float, L, 2> {
     static __device__ __forceinline__ void run(float T, float pref, float* F, const PairTable<float>& P)
     {
-        if (T < (float)MESS_BOYS_TMAX32) boys_small_f32<L>(T, F, P.boys32v); else boys_large_f32<L>(T, F);
+        boys_f32<L>(T, F, P.boys32v);
 #pragma unroll
         for (int m = 0; m <= L; ++m) F[m] *= pref;
     }
@@ -395,7 +394,7 @@ __device__ __forceinline__ void boys_eval(R T, R pref, R* F, const PairTable<R>&
 // 1/(zeta + eta) and its square root (the prefactor's 1/sqrt(zeta + eta)): one reciprocal square root and
 // its square, instead of a division and a root (FP64: 8 instructions of the FP64 pipe instead of about 20)
 __device__ __forceinline__ void recip_and_sqrt(double s, double& rz, double& sq) { sq = rsqrt(s); rz = sq * sq; }
-__device__ __forceinline__ void recip_and_sqrt(float s, float& rz, float& sq) { sq = rsqrtf(s); rz = sq * sq; }
+__device__ __forceinline__ void recip_and_sqrt(float s, float& rz, float& sq) { sq = rsqrt_ftz(s); rz = sq * sq; }
 __device__ __forceinline__ void recip_and_sqrt(df32 s, df32& rz, df32& sq) { sq = df_rsqrt(s); rz = sq * sq; }
 
 // primitive loops of the straight-line FP32 kernels run two primitive quartets per iteration (more

@@ -8,7 +8,7 @@
 #define MESS_BOYS_DT 0.1
 #define MESS_BOYS_TMAX64 48.0     // FP64: Taylor expansion below this
 #define MESS_BOYS_TMAXDF 36.0     // double-float, and the FP64 Boys function of FP32 quartets
-#define MESS_BOYS_TMAX32 30.0     // FP32 (Taylor order 4)
+#define MESS_BOYS_TMAX32 36.0     // FP32
 #define MESS_BOYS_NF 16
 #define MESS_BOYS_NCOL (MESS_BOYS_NF + 1)
 #define MESS_BOYS_NROW 362
@@ -21,13 +21,13 @@
 #define MESS_BOYS64_NROW 1538
 #define MESS_BOYSDF_INV_DT 64.0
 #define MESS_BOYSDF_NROW 2306
-// FP32 rows: T_k = k * MESS_BOYS32_DT with a step that FP32 holds exactly (1/16: T_k - T is then
-// formed with one rounding; a step of 0.1 or 0.05 rounded to FP32 shifts x by up to 5e-7 at the far
-// end of the grid, a one-signed error of up to 1e-7 in F_L); F_L, F_L+1, F_L+2 and exp(-T_k) in one
-// 16-byte row (Taylor order 4, F_L+3 and F_L+4 from the upward recursion); rows up to T = MESS_BOYS_TMAX32.
-#define MESS_BOYS32_DT 0.0625
-#define MESS_BOYS32_INV_DT 16.0
-#define MESS_BOYS32_NROW 482
+// FP32 rows: step 1/128, which FP32 holds exactly (T_k - T is then exact; a step of 0.1 or 0.05 rounded to
+// FP32 shifts x by up to 5e-7 at the far end of the grid, a one-signed error of up to 1e-7 in F_L).
+// F_L, F_L+1, F_L+2 / 2 and exp(-T_k) in one 16-byte row: order 2 leaves at most 8e-9 of F_L, of both signs.
+// L = 0, which needs no exp(-T): F_0, F_1, F_2 / 2, F_3 / 6 at a step of 1/32 (order 3 leaves 3e-10).
+#define MESS_BOYS32_INV_DT 128.0
+#define MESS_BOYS32_INV_DT0 32.0
+#define MESS_BOYS32_NROW 4610
 
 #define MESS_PRIM_EPS 1e-18       // primitive pairs below this weight bound are left out (build_pairs)
 

@@ -93,3 +93,50 @@ def test_double_float_scheme(oracle_mod):
         for L in (0, 1, 4, 8):
             Ts, got = _taylor_df(T, L, oracle_mod.boys)
             assert np.abs(np.array(got) / oracle_mod.boys(L, Ts) - 1).max() <= 1e-13, (T, L)
+
+
+def _scheme_f32(T, L, boys):
+    """The FP32 scheme: second-order expansion about k / 128 (third order about k / 32 for L = 0) and downward recursion
+    below 36, the asymptote without exp(-T) above."""
+    T = F(T)
+    rt = F(1.0 / math.sqrt(float(T))) if T > 0 else F(0)
+    if T >= F(36.0):
+        h, out = F(F(0.5) * rt * rt), [F(F(0.886226925) * rt)]
+        for m in range(L):
+            out.append(F(out[-1] * F(F(2 * m + 1) * h)))
+        return float(T), [float(v) for v in out]
+    fma = lambda a, b, c: F(float(a) * float(b) + float(c))
+    step = 128.0 if L else 32.0
+    k = int(np.rint(step * float(T)))
+    c, x = boys(L + 3, k / step), F(k / step - float(T))
+    assert float(x) == k / step - float(T)
+    d = fma(x, fma(x, F(0.5 * c[L + 2]) if L else fma(x, F(c[3] / 6), F(0.5 * c[2])), F(c[L + 1])), F(c[L]))
+    e = F(F(math.exp(-k / step)) * fma(x, fma(x, fma(x, F(1 / 6), F(0.5)), F(1)), F(1)))
+    out = [d]
+    for m in range(L, 0, -1):
+        d = F(fma(F(2) * T, d, e) * F(1.0 / (2 * m - 1)))
+        out.append(d)
+    return float(T), [float(v) for v in out[::-1]]
+
+
+def test_fp32_scheme(oracle_mod):
+    """Each order within its roundings (u = 2^-24): two of the table and expansion (and 8e-9 left out), 3 more per
+    step of the recursion; above the grid the root's and three per order.  The highest order drifts to
+    no side: every FP32 integral would inherit that."""
+    rng = np.random.default_rng(6)
+    u = 2.0 ** -24
+    near = np.concatenate([[0.0, 1e-9, 1.0 / 256, 35.999], rng.uniform(0, 36, 600), rng.uniform(0, 1, 100)])
+    for L in (0, 1, 2, 4, 8):
+        drift = []
+        for T in near:
+            Ts, got = _scheme_f32(T, L, oracle_mod.boys)
+            rel = np.array(got) / oracle_mod.boys(L, Ts) - 1
+            for m in range(L + 1):
+                assert abs(rel[m]) <= (3 + 3 * (L - m)) * u + 8e-9, (T, L, m, rel[m])
+            drift.append(rel[L])
+        assert abs(np.mean(drift)) < 6e-9, (L, np.mean(drift))
+        for T in (36.0, 36.5, 40.0, 90.0, 1e3, 1e4):
+            Ts, got = _scheme_f32(T, L, oracle_mod.boys)
+            rel = np.array(got) / oracle_mod.boys(L, Ts) - 1
+            for m in range(L + 1):
+                assert abs(rel[m]) <= (3 + 5 * m) * u + 1e-8, (T, L, m, rel[m])
