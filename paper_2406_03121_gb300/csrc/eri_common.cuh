@@ -468,6 +468,10 @@ __device__ __forceinline__ void jk_add(double* __restrict__ M, size_t idx, R v, 
         if (v != R(0)) atomicAdd(M + idx, to_f64(v));
     }
 }
+__device__ __forceinline__ void jk_add(double* __restrict__ M, size_t idx, df32u v, bool warp_reduce)
+{
+    jk_add<df32>(M, idx, v, warp_reduce);
+}
 
 // ------------------------------------------------------------------------------------------
 // Work decomposition of one class bin: bra pairs i (sorted by Q descending), each with a
