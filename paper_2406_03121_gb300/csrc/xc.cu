@@ -29,6 +29,7 @@ constexpr int kNTheta = 16, kNPhi = 32;
 constexpr int kFuncThreads = 128;                   // points per block of the functional
 constexpr int kVxcThreads = 256, kVxcTile = 64;     // threads and function tile of the V_xc reduction
 constexpr int kVxcMaxEl = kVxcTile * kVxcTile / kVxcThreads;   // elements per thread at most
+constexpr int kSmallN = 4;                            // functions up to which V_xc is summed by the functional
 constexpr int kLogBins = 128;                       // entries of the logarithm table
 constexpr double kRhoMin = 1e-14;   // points with less density carry no exchange-correlation energy
 
@@ -281,26 +282,41 @@ struct FuncArgs {
     double* vgrad;           // [npts][3] w * 2 d e / d sigma * grad rho (PBE)
     const double2* logs;     // table of log_1p
     double* Exc;             // [nmol] accumulated
+    double* V;               // packed, accumulated (N > 0)
+    int ppt;                 // points per thread
 };
 
-// density, its gradient, and the functional at every point of a molecule (grid.y = molecule, one
-// thread per point); E_xc accumulated per molecule.
+// density, its gradient, and the functional at every point of a molecule (grid.y = molecule, ppt points
+// per thread); E_xc accumulated per molecule.  N > 0: the molecules have at most N functions, and the
+// kernel adds V_xc as well (see k_vxc): a point's phi and v_rho are in its registers already, and N (N + 1) / 2
+// sums per thread fit there.  N = 0: v_rho and v_sigma grad rho go to memory for k_vxc.
 // Bound: the FP64 pipe (two FMA lanes per SM and clock): n^2 FMAs per point for D phi and about 80
 // (LDA) to 170 (PBE) instructions of the functional.  So the memory side only has to stay out of the
 // way: phi function by function (coalesced, re-read from L1), D as warp-uniform loads, four rows of D
 // per pass so that four accumulation chains hide the FMA latency.  The functional works from
 // rho^(-1/3) and multiplies where it can.  CH4 / 6-31G / PBE (17 functions, 140,800 points): 231 -> 155 us
 // (167 with the library's roots and logarithms); 64 H2 (51,200 points each), LDA: 729 -> 445 us (546).
-template <int KIND>
+// With V_xc in it (N = 2), 480 us instead of 445 and k_vxc's 148; minimisation of 64 H2, 128 steps: STO-3G 95.0 ->
+// 79.6 ms in LDA, 187 -> 177 in PBE; 6-31G (N = 4) 124 -> 104 and 224 -> 218.  Beyond four functions the sums of
+// a thread outgrow its registers in PBE.
+template <int KIND, int N>
 __global__ void __launch_bounds__(kFuncThreads) k_functional(FuncArgs f)
 {
-    __shared__ double red[kFuncThreads / 32];
+    constexpr int NS = 1 + N * (N + 1) / 2;             // sums of a thread: E_xc, V_ij (i <= j)
+    __shared__ double red[kFuncThreads / 32][NS];
     const int m = blockIdx.y, n = f.mn[m];
     const long long np_ = f.pbase[m + 1] - f.pbase[m];
-    if ((long long)blockIdx.x * kFuncThreads >= np_) return;
-    const long long lp = (long long)blockIdx.x * kFuncThreads + threadIdx.x;
-    double e = 0.0;
-    if (lp < np_) {
+    const long long first = (long long)blockIdx.x * kFuncThreads * f.ppt;
+    if (first >= np_) return;
+    double sum[NS], Dr[N > 0 ? N * N : 1];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) sum[k] = 0.0;
+#pragma unroll
+    for (int k = 0; k < N * N; ++k) Dr[k] = k / N < n && k % N < n ? __ldg(f.D + f.mbase[m] + k / N * n + k % N) : 0.0;
+    for (int pt = 0; pt < f.ppt; ++pt) {
+        const long long lp = first + pt * kFuncThreads + threadIdx.x;
+        if (lp >= np_) break;
+        double e = 0.0, pv[N > 0 ? N : 1], dv[KIND == 2 && N > 0 ? 3 * N : 1];
         const double* ph = f.phi + f.aobase[m] + lp;
         const double* dx = f.dphi + 3 * f.aobase[m] + lp;
         const double* dy = dx + np_ * n;
@@ -315,7 +331,28 @@ __global__ void __launch_bounds__(kFuncThreads) k_functional(FuncArgs f)
                 gz += 2.0 * t * dz[i * np_];
             }
         };
-        int i = 0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            pv[k] = k < n ? ph[k * np_] : 0.0;
+            if (KIND == 2) {
+                dv[3 * k] = k < n ? dx[k * np_] : 0.0;
+                dv[3 * k + 1] = k < n ? dy[k * np_] : 0.0;
+                dv[3 * k + 2] = k < n ? dz[k * np_] : 0.0;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            double t = 0.0;
+#pragma unroll
+            for (int j = 0; j < N; ++j) t += Dr[k * N + j] * pv[j];
+            rho += t * pv[k];
+            if (KIND == 2) {
+                gx += 2.0 * t * dv[3 * k];
+                gy += 2.0 * t * dv[3 * k + 1];
+                gz += 2.0 * t * dv[3 * k + 2];
+            }
+        }
+        int i = N > 0 ? n : 0;
         for (; i + 4 <= n; i += 4) {
             const double* D0 = D + (long long)i * n;
             double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
@@ -386,21 +423,54 @@ __global__ void __launch_bounds__(kFuncThreads) k_functional(FuncArgs f)
         }
         const long long p = f.pbase[m] + lp;
         const double w = f.w[p];
-        e *= w;
-        f.vrho[p] = w * vr;
-        if (KIND == 2) {
-            f.vgrad[3 * p] = w * 2.0 * vs * gx;
-            f.vgrad[3 * p + 1] = w * 2.0 * vs * gy;
-            f.vgrad[3 * p + 2] = w * 2.0 * vs * gz;
+        sum[0] += e * w;
+        if (N > 0) {
+            double a[N > 0 ? N : 1];                    // LDA: w v_rho phi; PBE: half of it, and the gradient's part
+            const double ws = w * 2.0 * vs, wr = (KIND == 2 ? 0.5 : 1.0) * w * vr;
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                a[k] = wr * pv[k];
+                if (KIND == 2) a[k] += ws * (gx * dv[3 * k] + gy * dv[3 * k + 1] + gz * dv[3 * k + 2]);
+            }
+#pragma unroll
+            for (int c = 0; c < N; ++c)
+#pragma unroll
+                for (int r = 0; r <= c; ++r) {
+                    double& v = sum[1 + c * (c + 1) / 2 + r];
+                    v += a[r] * pv[c];
+                    if (KIND == 2) v += pv[r] * a[c];
+                }
+        } else {
+            f.vrho[p] = w * vr;
+            if (KIND == 2) {
+                f.vgrad[3 * p] = w * 2.0 * vs * gx;
+                f.vgrad[3 * p + 1] = w * 2.0 * vs * gy;
+                f.vgrad[3 * p + 2] = w * 2.0 * vs * gz;
+            }
         }
     }
-    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        for (int o = 16; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = sum[k];
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    const int k = threadIdx.x;
+    if (k < NS) {
         double t = 0.0;
-        for (int k = 0; k < kFuncThreads / 32; ++k) t += red[k];
-        atomicAdd(f.Exc + m, t);
+        for (int g = 0; g < kFuncThreads / 32; ++g) t += red[g][k];
+        if (k == 0) {
+            atomicAdd(f.Exc + m, t);
+        } else {
+            int c = 0;
+            while ((c + 1) * (c + 2) / 2 <= k - 1) ++c;
+            const int r = k - 1 - c * (c + 1) / 2;
+            if (c < n) {
+                double* V = f.V + f.mbase[m];
+                atomicAdd(V + (long long)r * n + c, t);
+                if (r != c) atomicAdd(V + (long long)c * n + r, t);
+            }
+        }
     }
 }
 
@@ -418,8 +488,9 @@ struct VxcArgs {
     double* V;               // packed, accumulated
 };
 
+// (molecules of more than kSmallN functions)
 // V_mn += sum over a chunk of the molecule's points of a_m phi_n + phi_m a_n, a = (1/2) w v_rho phi +
-// w 2 v_sigma grad rho . grad phi (vgrad holds w 2 v_sigma grad rho); grid (chunks, tile pairs, nmol).
+// w 2 v_sigma grad rho . grad phi (vgrad holds w 2 v_sigma grad rho); LDA: of w v_rho phi_m phi_n; grid (chunks, tile pairs, nmol).
 // A block owns the elements m <= n of one pair of kVxcTile x kVxcTile function tiles.  It stages phi and
 // a of tp points at a time in shared memory (a is formed once per function and point) and every thread
 // sums its elements over the points.  Where a tile pair has fewer elements than threads (H2: 3), groups
@@ -487,7 +558,7 @@ __global__ void __launch_bounds__(kVxcThreads) k_vxc(VxcArgs v)
             if (p < cnt) {
                 const long long at = (long long)(r < ni ? i0 + r : j0 + r - rj) * np_ + p0 + p;
                 fv = ph[at];
-                av = 0.5 * v.vrho[gp + p0 + p] * fv;
+                av = (KIND == 2 ? 0.5 : 1.0) * v.vrho[gp + p0 + p] * fv;
                 if (KIND == 2) {
                     const double* g = v.vgrad + 3 * (gp + p0 + p);
                     av += g[0] * dx[at] + g[1] * dy[at] + g[2] * dz[at];
@@ -505,7 +576,7 @@ __global__ void __launch_bounds__(kVxcThreads) k_vxc(VxcArgs v)
             double s0 = 0.0, s1 = 0.0;
             for (int p = grp; p < cnt; p += ngrp) {
                 s0 += ai[p] * fj[p];
-                s1 += fi[p] * aj[p];
+                if (KIND == 2) s1 += fi[p] * aj[p];      // (LDA: the same as s0, in a)
             }
             acc[k] += s0 + s1;
         }
@@ -650,11 +721,18 @@ mess_status mess_xc_eval(mess_basis* b, int kind, const double* dD, double* dV, 
     MESS_CUDA_TRY(cudaMemsetAsync(dV, 0, sizeof(double) * b->packed, s));
     if (X.npts == 0) return MESS_OK;
     FuncArgs f{X.phi.p, X.dphi.p, dD, b->d_mol_base.p, X.pbase.p, X.aobase.p, b->d_mol_n.p, X.w.p, X.vrho.p, X.vgrad.p,
-               reinterpret_cast<const double2*>(X.tab.p), dExc};
-    const dim3 fgrid((unsigned)((X.mol_npts_max + kFuncThreads - 1) / kFuncThreads), (unsigned)b->nmol);
-    if (kind == 2) k_functional<2><<<fgrid, kFuncThreads, 0, s>>>(f);
-    else k_functional<1><<<fgrid, kFuncThreads, 0, s>>>(f);
+               reinterpret_cast<const double2*>(X.tab.p), dExc, dV, 1};
+    // sixteen blocks per SM before a thread takes more points (fewer sums over a block's threads)
+    f.ppt = (int)std::clamp<long long>(X.npts / (152LL * 16 * kFuncThreads), 1, 8);
+    const dim3 fgrid((unsigned)((X.mol_npts_max + (long long)kFuncThreads * f.ppt - 1) / ((long long)kFuncThreads * f.ppt)), (unsigned)b->nmol);
+    typedef void (*Kernel)(FuncArgs);
+    static const Kernel kernels[2][kSmallN + 1] = {
+        {k_functional<1, 0>, k_functional<1, 1>, k_functional<1, 2>, k_functional<1, 3>, k_functional<1, 4>},
+        {k_functional<2, 0>, k_functional<2, 1>, k_functional<2, 2>, k_functional<2, 3>, k_functional<2, 4>}};
+    const int small_n = b->max_nbf <= kSmallN ? b->max_nbf : 0;
+    kernels[kind - 1][small_n]<<<fgrid, kFuncThreads, 0, s>>>(f);
     MESS_CUDA_TRY(cudaGetLastError());
+    if (small_n) return MESS_OK;
     // V_xc: function tiles of the largest molecule; points staged per pass so that phi and a of the
     // staged functions take at most about 40 KB (16 to 256 points, fewer where functions are many);
     // about eight blocks per SM over all molecules and tile pairs, each with enough points to pay for
