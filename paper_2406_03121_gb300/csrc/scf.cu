@@ -608,6 +608,39 @@ struct StreamGuard {
     }
 };
 
+// A second stream beside a call's own, for work that needs what the call's stream has produced up to begin() and
+// is needed after join(); without create() that work runs on the call's stream.  Drained before the buffers
+// declared ahead of it are freed.
+struct SideStream {
+    StreamGuard g;
+    cudaEvent_t fork = nullptr, done = nullptr;
+    ~SideStream()
+    {
+        if (fork) cudaEventDestroy(fork);
+        if (done) cudaEventDestroy(done);
+    }
+    cudaError_t create()
+    {
+        cudaError_t e = cudaStreamCreateWithFlags(&g.s, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+        return e;
+    }
+    cudaError_t begin(cudaStream_t main, cudaStream_t* use)
+    {
+        *use = g.s ? g.s : main;
+        if (!g.s) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(fork, main);
+        return e == cudaSuccess ? cudaStreamWaitEvent(g.s, fork, 0) : e;
+    }
+    cudaError_t join(cudaStream_t main)
+    {
+        if (!g.s) return cudaSuccess;
+        const cudaError_t e = cudaEventRecord(done, g.s);
+        return e == cudaSuccess ? cudaStreamWaitEvent(main, done, 0) : e;
+    }
+};
+
 struct SCFState {
     mess_basis* b;
     cudaStream_t s;
@@ -983,11 +1016,21 @@ mess_status scf_run(mess_basis* b, const mess_scf_opts* opts, mess_scf_result* r
         mess_status xs = mess_xc_prepare(b, st.s);
         if (xs != MESS_OK) return xs;
     }
+    // V_xc and E_xc of the density, beside the J/K build: few FP64 quartets leave most of the GPU idle.  PBE SCF of
+    // H2O / 6-31G* 10.2 -> 9.1 ms, CH4 / 6-31G 9.85 -> 9.3, four waters 256 -> 250.  With one part of quartets
+    // (H2 / STO-3G, 1.10 -> 1.17 ms) the stream costs more than it hides.
+    SideStream side;
+    if (o.xc && b->bins.parts.size() > 1) MESS_CUDA_TRY(side.create());
+    auto xc_begin = [&]() -> mess_status {
+        if (!o.xc) return MESS_OK;
+        cudaStream_t xs = nullptr;
+        MESS_CUDA_TRY(side.begin(st.s, &xs));
+        return mess_xc_eval(b, o.xc, st.D.p, Vxc.p, Exc.p, xs);
+    };
     // F = H + J - K/2 (Hartree-Fock) or H + J + V_xc (Kohn-Sham) from the accumulated J, K, and its energy
     auto fock_energy = [&]() -> mess_status {
         if (o.xc) {
-            mess_status xs = mess_xc_eval(b, o.xc, st.D.p, Vxc.p, Exc.p, st.s);
-            if (xs != MESS_OK) return xs;
+            MESS_CUDA_TRY(side.join(st.s));
             k_axpbypcz<<<eg, 256, 0, st.s>>>(st.F.p, 1.0, st.H.p, 1.0, st.Jt.p, 1.0, Vxc.p, st.L);
             k_energy_ks<<<b->nmol, 256, 0, st.s>>>(st.D.p, st.H.p, st.Jt.p, Exc.p, st.L, st.E.p);
         } else {
@@ -1035,7 +1078,9 @@ mess_status scf_run(mess_basis* b, const mess_scf_opts* opts, mess_scf_result* r
                                                                    b->d_shell_f0.p, b->d_shell_l.p, dmax.p, b->npair);
             MESS_CUDA_TRY(cudaGetLastError());
         }
-        mess_status js = mess_jk_enqueue_only(b, st.W1.p, st.J.p, st.K.p, &jo);
+        mess_status js = xc_begin();
+        if (js != MESS_OK) return js;
+        js = mess_jk_enqueue_only(b, st.W1.p, st.J.p, st.K.p, &jo);
         if (js != MESS_OK) return js;
         k_axpbypcz<<<eg, 256, 0, st.s>>>(st.Jt.p, 1.0, st.Jt.p, 1.0, st.J.p, 0.0, nullptr, st.L);
         k_axpbypcz<<<eg, 256, 0, st.s>>>(st.Kt.p, 1.0, st.Kt.p, 1.0, st.K.p, 0.0, nullptr, st.L);
@@ -1175,7 +1220,9 @@ mess_status scf_run(mess_basis* b, const mess_scf_opts* opts, mess_scf_result* r
         // ten times more of the largest quartets in FP64-class arithmetic than in the iterations
         const double it_tau = o.prec == MESS_MIXED ? (o.fp64_tau > 0.0 ? o.fp64_tau : MESS_DEFAULT_FP64_TAU) : 0.0;
         jf.fp64_tau = it_tau > 0.0 ? 0.1 * it_tau : 1e-300;
-        mess_status js = mess_jk_packed(b, st.D.p, st.Jt.p, st.Kt.p, &jf, nullptr);
+        mess_status js = xc_begin();
+        if (js != MESS_OK) return js;
+        js = mess_jk_packed(b, st.D.p, st.Jt.p, st.Kt.p, &jf, nullptr);
         if (js != MESS_OK) return js;
         js = fock_energy();
         if (js != MESS_OK) return js;
@@ -1419,17 +1466,29 @@ mess_status min_run(mess_basis* b, const mess_min_opts* opts, mess_scf_result* r
     jo.boys_fp64 = o.boys_fp64;
     jo.split_df32 = o.split_df32;
     jo.cuda_stream = st.s;
+    SideStream side;                                                         // V_xc beside the J/K build, as in the SCF
+    if (o.xc) {
+        const mess_status bs = mess_jk_ensure_bins(b, &jo);
+        if (bs != MESS_OK) return bs;
+        if (b->bins.parts.size() > 1) MESS_CUDA_TRY(side.create());
+    }
     // E(Z) on every molecule (trace row `row`), and with grad = true dE/dZ into G
     auto energy = [&](int row, bool grad) -> mess_status {
         k_qr<<<nmol, 256, 0, st.s>>>(Z.p, Q.p, R.p, Vh.p, st.L, singular.p);
         MESS_CUDA_TRY(cudaGetLastError());
         MESS_CUDA_TRY(gemm(st, false, st.X.p, Q.p, st.C.p, 0, 1.0));        // C = X Q
         MESS_CUDA_TRY(gemm(st, true, st.C.p, st.C.p, st.D.p, 1, 1.0));      // D = C diag(occ) C^T
-        mess_status js = mess_jk_packed(b, st.D.p, st.J.p, st.K.p, &jo, nullptr);
+        mess_status js = MESS_OK;
+        if (o.xc) {
+            cudaStream_t xs = nullptr;
+            MESS_CUDA_TRY(side.begin(st.s, &xs));
+            js = mess_xc_eval(b, o.xc, st.D.p, Vxc.p, Exc.p, xs);
+            if (js != MESS_OK) return js;
+        }
+        js = mess_jk_packed(b, st.D.p, st.J.p, st.K.p, &jo, nullptr);
         if (js != MESS_OK) return js;
         if (o.xc) {                                                          // F = H + J + V_xc (Kohn-Sham)
-            js = mess_xc_eval(b, o.xc, st.D.p, Vxc.p, Exc.p, st.s);
-            if (js != MESS_OK) return js;
+            MESS_CUDA_TRY(side.join(st.s));
             k_axpbypcz<<<eg, 256, 0, st.s>>>(st.F.p, 1.0, st.H.p, 1.0, st.J.p, 1.0, Vxc.p, st.L);
             k_energy_ks<<<nmol, 256, 0, st.s>>>(st.D.p, st.H.p, st.J.p, Exc.p, st.L, st.E.p);
         } else {                                                             // F = H + J - K/2
