@@ -917,7 +917,7 @@ __device__ __forceinline__ const R* team_eri(const PairTable<R>& P, int bp, cons
     const int k0 = kv.k0, nkp = kv.nk;
     const R ACx = kv.AC[0], ACy = kv.AC[1], ACz = kv.AC[2];
 #pragma unroll 1
-    for (int ip = PS ? pslot : 0; ip < nbp * nkp; ip += PS ? MESS_TEAM_WARPS : 1) {
+    for (int ip = PS ? pslot + MESS_TEAM_WARPS * (int)blockIdx.y : 0; ip < nbp * nkp; ip += PS ? MESS_TEAM_WARPS * (int)gridDim.y : 1) {
         const int ib = b0 + ip / nkp, ik = k0 + ip % nkp;
         const PrimPair<R> pb = P.load(ib);
         {

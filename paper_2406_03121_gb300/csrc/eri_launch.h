@@ -1,5 +1,7 @@
 // Host-side launch interface of the generated per-class ERI kernels.
 #pragma once
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "df32.cuh"
@@ -16,8 +18,9 @@ enum { MESS_MODE_FP64 = 0, MESS_MODE_MIXED = 1, MESS_MODE_FP32 = 2, MESS_MODE_DF
 struct ClassLaunchArgs {
     int kind;                    // MESS_KIND_*
     int mode;                    // MESS_MODE_* (JK only)
-    int G;                       // JK: lanes per shell quartet (1, 4 or 8)
+    int G;                       // JK: lanes per shell quartet (1, 4, 8 or 32)
     int team;                    // JK: 1 = one warp per shell quartet (level-scheduled program)
+    int split;                   // JK: blocks that share a quartet's primitive quartets (G = 32, team 3; 0: one)
     BinLaunch bin;               // JK / STORE
     const RunLaunch* runs;       // JK: the FP32 one-thread kernel goes by bra runs (null: by quartets)
     const int* pairs;            // SCHWARZ: pair ids of one diagonal class
@@ -51,6 +54,24 @@ inline int schwarz_lanes(int npairs)
 {
     const long long fill = 152LL * 4 * 32;
     return npairs >= fill ? 1 : (8LL * npairs >= fill ? 8 : 32);
+}
+
+// Blocks over which the primitive quartets of a part's shell quartets are split (the J/K digestion is linear in
+// the integrals, so each block adds its share's): the quartets of a part on a warp (G = 32) or a block
+// (team 3) each run their primitive quartets as one chain, which a part of fewer quartets than SMs
+// leaves on a few of them.  At most two blocks per SM, and a full pass of lanes each.  Only where the whole build
+// has few quartets: otherwise the other parts fill the SMs, and the repeated HRR and digestion cost more
+// (kMaxBuild lies between one water / 6-31G, 1,035 quartets, 98 -> 76 us, and C2H6 / 6-31G*, 45,000, 352 -> 367).
+// One water / STO-3G in FP64: (pp|pp), one quartet of 81 primitive quartets, 80 -> 45 us, (pp|ps) 31 -> 18, the
+// whole call 115 -> 80.
+inline int prim_split(long long quartets, long long prim_quartets, int G, int team, long long build_quartets)
+{
+    constexpr long long kMaxBuild = 16384;
+    if (build_quartets > kMaxBuild) return 1;
+    const int lanes = team == 3 ? MESS_TEAM_WARPS : (G == 32 && !team ? 32 : 0);
+    if (!lanes || quartets <= 0 || quartets > 152) return 1;
+    const long long passes = (prim_quartets / quartets + lanes - 1) / lanes;
+    return (int)std::max(1LL, std::min(passes, 2 * 152 / quartets));
 }
 
 typedef cudaError_t (*mess_class_launcher)(const ClassLaunchArgs&);

@@ -634,7 +634,8 @@ def emit_class_straight(cls):
     lines.append("    }")
     lines.append("    } else {")
     lines.append("    // the G lanes of a group split the primitive quartets (flattened index g, g + G, ...)")
-    lines.append("    int ib = b0, ik = k0 + g;")
+    lines.append("    // of the blocks that split them further (prim_split)")
+    lines.append("    int ib = b0, ik = k0 + g + (G == 32 ? G * (int)blockIdx.y : 0);")
     lines.append("    while (ik >= k1 && ib < b1) { ik -= nk; ++ib; }")
     lines.append("#pragma unroll 1")
     lines.append("    while (ib < b1) {")
@@ -643,7 +644,7 @@ def emit_class_straight(cls):
     lines.append("            const PrimPair<R> pk = P.load(ik);")
     lines += body
     lines.append("        }")
-    lines.append("        ik += G;")
+    lines.append("        ik += G == 32 ? G * (int)gridDim.y : G;")
     lines.append("        while (ik >= k1 && ib < b1) { ik -= nk; ++ib; }")
     lines.append("    }")
     lines.append(f"    GroupSums<G / 2, {nacc}>::run(acc, g, 0, {nacc}, sh);")
@@ -1013,7 +1014,7 @@ def main(outdir):
               "        const int qpb = a.team >= 2 ? 1 : MESS_TEAM_WARPS;",
               "        const long long nbt = (a.bin.total + qpb - 1) / qpb;",
               "        if (nbt > 0x7fffffffLL) return cudaErrorInvalidConfiguration;",
-              "        const dim3 gt((unsigned)nbt);",
+              "        const dim3 gt((unsigned)nbt, a.team == 3 ? (unsigned)std::max(1, a.split) : 1);",
               "        if (a.team == 3) {",
               "            if (a.mode == MESS_MODE_FP64)",
               f"                return mess_team_launch<double, 0>(k_jk_team_{t}<double, 0, 32 * MESS_TEAM_WARPS, 1>, gt, team_smem_{t}<double>(), a, *a.P64_ptr, cfg[8]);",
@@ -1049,7 +1050,7 @@ def main(outdir):
               f"            const int TG = jk_block_threads(a.bin.total * {GG});",
               f"            const long long nbg = (a.bin.total * {GG} + TG - 1) / TG;",
               "            if (nbg > 0x7fffffffLL) return cudaErrorInvalidConfiguration;",
-              "            const dim3 gg((unsigned)nbg);",
+              f"            const dim3 gg((unsigned)nbg, {'(unsigned)std::max(1, a.split)' if GG == 32 else '1'});",
               "            if (a.mode == MESS_MODE_FP64)",
               f"                k_jk_{t}<double, 0, {GG}><<<gg, TG, 0, a.stream>>>(a.bin, *a.P64_ptr, dmat<double>(a), a.J, a.K, a.n);",
               "            else if (a.mode == MESS_MODE_MIXED)",

@@ -177,6 +177,7 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
     BinSet& B = b->bins;
     if (B.tau == tau && B.tau64 == tau64 && B.split == split && B.active_version == b->active_version) return MESS_OK;
     B.parts.clear();
+    B.total = 0;
     // per ket list (pair class x primitive group): Q, and prefix sums of unique function pairs and of
     // primitive pairs, in list order
     const int NL = MESS_NLIST;
@@ -335,6 +336,7 @@ mess_status mess_ensure_bins(mess_basis* b, double tau, double tau64, int split)
             bp.run_offs_off += offs.size();
             bp.run_off += run.size();
             B.parts.push_back(bp);
+            B.total += bp.total;
         }
         run.insert(run.end(), T.run.begin(), T.run.end());
         bra.insert(bra.end(), T.bra.begin(), T.bra.end());
@@ -1158,6 +1160,7 @@ static mess_status jk_enqueue(mess_basis* b, const mess_jk_opts& o, const double
         a.bin = bin_launch(b, p);
         const RunLaunch runs = run_launch(b, p);
         a.runs = by_runs(p, a.G, a.team, a.mode) ? &runs : nullptr;
+        a.split = prim_split(p.total, p.prim_quartets, a.G, a.team, b->bins.total);
         a.P64_ptr = &b->P64;
         a.P32_ptr = &b->P32;
         a.Pdf_ptr = &b->Pdf;
@@ -1493,6 +1496,7 @@ static mess_status jk_autotune_device(mess_basis* b, const double* dD, double* d
             a.bin = bin_launch(b, p);
             const RunLaunch runs = run_launch(b, p);
             a.runs = by_runs(p, v.G, v.team, v.mode) ? &runs : nullptr;
+            a.split = prim_split(p.total, p.prim_quartets, v.G, v.team, b->bins.total);
             a.P64_ptr = &b->P64;
             a.P32_ptr = &b->P32;
             a.Pdf_ptr = &b->Pdf;

@@ -94,6 +94,7 @@ struct BinSet {
     long long active_version = -1;
     long long generation = 0;   // incremented on every rebuild (cached graphs refer to one generation)
     std::vector<BinPart> parts;
+    long long total = 0;        // shell quartets of all parts
     DevBuf<int> bra, kbeg;
     DevBuf<long long> offs;
     DevBuf<int> seg;
