@@ -40,9 +40,11 @@ template <typename T> struct DevBuf {
     cudaError_t alloc(size_t count)
     {
         free();
-        n = count;
         if (count == 0) return cudaSuccess;
-        return cudaMalloc((void**)&p, count * sizeof(T));
+        const cudaError_t e = cudaMalloc((void**)&p, count * sizeof(T));
+        if (e == cudaSuccess) n = count;   // (callers that keep a buffer ask n whether it is large enough)
+        else p = nullptr;
+        return e;
     }
     cudaError_t upload(const std::vector<T>& h)
     {
