@@ -457,6 +457,7 @@ namespace {
 cudaError_t ensure_cap(mess_mlp* m, long long rows)
 {
     if (rows <= m->cap) return cudaSuccess;
+    m->cap = 0;                                 // until every buffer is there: a later call starts over
     cudaError_t e;
     if ((e = m->xb.alloc(rows * DIN)) != cudaSuccess) return e;
     if ((e = m->a1.alloc(rows * WID)) != cudaSuccess) return e;

@@ -30,3 +30,8 @@ def test_the_input_buffer_is_allocated_again(mess, lines):
     k, large, small, whole = _passes(lines)[0]
     assert (large, small, whole) == (mess.MESS_ENOMEM, mess.MESS_OK, 1)
     assert "null 0" in lines
+
+
+def test_the_activation_buffers_are_allocated_again(mess, lines):
+    for k, large, small, whole in _passes(lines)[1:]:
+        assert (large, small, whole) == (mess.MESS_ENOMEM, mess.MESS_OK, 1), k
