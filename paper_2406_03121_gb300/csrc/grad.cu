@@ -243,6 +243,7 @@ extern "C" mess_status mess_gradient(const mess_basis* bc, const mess_scf_opts* 
     }
     DevBuf<double> dD, dW, De, Se, Te, Ve, He, Je, Ke, VA, dg, drc, dlc;
     DevBuf<int> dfatom, dridx, dlidx;
+    const StreamDrain drain{(cudaStream_t)o.cuda_stream};
     MESS_CUDA_TRY(dD.upload(Dh));
     MESS_CUDA_TRY(dW.alloc(nn));
     for (DevBuf<double>* d : {&De, &Se, &Te, &Ve, &He, &Je, &Ke}) MESS_CUDA_TRY(d->alloc(ee));

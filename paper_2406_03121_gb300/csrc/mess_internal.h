@@ -33,10 +33,14 @@ struct PhaseTimer {
         }                                                                                         \
     } while (0)
 
-// A device allocation owned by the basis.
+// A device allocation, given back when its owner (a basis, a network, a call) goes.
 template <typename T> struct DevBuf {
     T* p = nullptr;
     size_t n = 0;
+    DevBuf() = default;
+    DevBuf(const DevBuf&) = delete;
+    DevBuf& operator=(const DevBuf&) = delete;
+    ~DevBuf() { free(); }
     cudaError_t alloc(size_t count)
     {
         free();
@@ -58,6 +62,12 @@ template <typename T> struct DevBuf {
         p = nullptr;
         n = 0;
     }
+};
+
+// Declared after a call's buffers: what the call has enqueued is done before they go, however it returns.
+struct StreamDrain {
+    cudaStream_t s;
+    ~StreamDrain() { cudaStreamSynchronize(s); }
 };
 
 struct HostShell {

@@ -647,13 +647,6 @@ mess_status init_params(mess_mlp* m, unsigned long long seed)
     return MESS_OK;
 }
 
-void free_mlp(mess_mlp* m)
-{
-    for (DevBuf<float>* d : {&m->w, &m->g, &m->m1, &m->m2, &m->z1, &m->z2, &m->y, &m->in}) d->free();
-    for (DevBuf<__nv_bfloat16>* d : {&m->wb, &m->xb, &m->a1, &m->a2, &m->dyb, &m->dz2, &m->dz1}) d->free();
-    m->loss.free();
-}
-
 // the rows' descriptors of a basis into X (device, rows x DIN); with D (device, packed) also targets
 mess_status features(const mess_basis* b, const AtomTables& t, const double* dD, float* X, float* T, float* M, cudaStream_t s)
 {
@@ -674,6 +667,7 @@ mess_status mess_mlp_guess_device(const mess_mlp* mc, const mess_basis* b, doubl
     mess_status st = atom_tables(b, t);
     if (st != MESS_OK) return st;
     DevBuf<float> X;
+    const StreamDrain drain{s};
     MESS_CUDA_TRY(X.alloc(t.rows * DIN));
     st = features(b, t, nullptr, X.p, nullptr, nullptr, s);
     if (st != MESS_OK) return st;
@@ -696,15 +690,13 @@ extern "C" mess_status mess_mlp_create(unsigned long long seed, mess_mlp** out)
     mess_mlp* m = new (std::nothrow) mess_mlp();
     if (!m) { mess_set_error("host allocation failed"); return MESS_ENOMEM; }
     mess_status st = init_params(m, seed);
-    if (st != MESS_OK) { free_mlp(m); delete m; return st; }
+    if (st != MESS_OK) { delete m; return st; }
     *out = m;
     return MESS_OK;
 }
 
 extern "C" void mess_mlp_destroy(mess_mlp* m)
 {
-    if (!m) return;
-    free_mlp(m);
     delete m;
 }
 
@@ -775,6 +767,7 @@ extern "C" mess_status mess_mlp_features(const mess_basis* b, const double* D, f
     if (D && (!T || !M)) { mess_set_error("targets need T and M"); return MESS_EINVAL; }
     DevBuf<float> dX, dT, dM;
     DevBuf<double> dD;
+    const StreamDrain drain{0};
     MESS_CUDA_TRY(dX.alloc(t.rows * DIN));
     if (D) {
         MESS_CUDA_TRY(dT.alloc(t.rows * DOUT));
@@ -835,6 +828,7 @@ extern "C" mess_status mess_mlp_train(mess_mlp* m, int nmol, mess_basis* const* 
     if (st != MESS_OK && st != MESS_ENOCONV) return st;
     DevBuf<float> X, T, M, Xb, Tb, Mb;
     DevBuf<long long> idx;
+    const StreamDrain drain{0};
     const long long rows = t.rows;
     MESS_CUDA_TRY(X.alloc(rows * DIN));
     MESS_CUDA_TRY(T.alloc(rows * DOUT));

@@ -35,3 +35,7 @@ def test_the_input_buffer_is_allocated_again(mess, lines):
 def test_the_activation_buffers_are_allocated_again(mess, lines):
     for k, large, small, whole in _passes(lines)[1:]:
         assert (large, small, whole) == (mess.MESS_ENOMEM, mess.MESS_OK, 1), k
+
+
+def test_a_destroyed_network_holds_nothing(lines):
+    assert "held 0" in lines
