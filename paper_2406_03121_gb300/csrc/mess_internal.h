@@ -33,6 +33,15 @@ struct PhaseTimer {
         }                                                                                         \
     } while (0)
 
+// cudaMalloc.  A failure is reported once, here: left as the runtime's last error, the next call's first launch
+// check would find it again.
+inline cudaError_t mess_device_alloc(void** p, size_t bytes)
+{
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) { *p = nullptr; cudaGetLastError(); }
+    return e;
+}
+
 // A device allocation, given back when its owner (a basis, a network, a call) goes.
 template <typename T> struct DevBuf {
     T* p = nullptr;
@@ -45,9 +54,8 @@ template <typename T> struct DevBuf {
     {
         free();
         if (count == 0) return cudaSuccess;
-        const cudaError_t e = cudaMalloc((void**)&p, count * sizeof(T));
+        const cudaError_t e = mess_device_alloc((void**)&p, count * sizeof(T));
         if (e == cudaSuccess) n = count;   // (callers that keep a buffer ask n whether it is large enough)
-        else p = nullptr;
         return e;
     }
     cudaError_t upload(const std::vector<T>& h)

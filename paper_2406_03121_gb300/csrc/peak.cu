@@ -29,7 +29,7 @@ cudaError_t time_fma(int iters, cudaStream_t s, double* tflops)
     if (e != cudaSuccess) return e;
     const int T = 256, B = nsm * 8;
     R* out = nullptr;
-    e = cudaMalloc((void**)&out, sizeof(R) * (size_t)T * B);
+    e = mess_device_alloc((void**)&out, sizeof(R) * (size_t)T * B);
     if (e != cudaSuccess) return e;
     cudaEvent_t t0, t1;
     cudaEventCreate(&t0);

@@ -596,7 +596,7 @@ __global__ void k_scale_cols(const double* __restrict__ U, const double* __restr
 
 template <typename T> struct Dev {
     T* p = nullptr;
-    cudaError_t alloc(size_t n) { return cudaMalloc((void**)&p, std::max<size_t>(n, 1) * sizeof(T)); }
+    cudaError_t alloc(size_t n) { return mess_device_alloc((void**)&p, std::max<size_t>(n, 1) * sizeof(T)); }
     ~Dev() { if (p) cudaFree(p); }
 };
 

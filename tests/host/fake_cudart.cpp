@@ -6,6 +6,7 @@
 
 long fake_fail_in = -1;      // allocations until one fails (-1: none)
 long fake_null_copies = 0;   // copies and fills that met a null pointer
+static int last_error = 0;   // as the runtime keeps it: until someone asks
 static std::set<void*>& live() { static std::set<void*> s; return s; }
 size_t fake_live() { return live().size(); }
 
@@ -15,7 +16,7 @@ struct Dim { unsigned x, y, z; };
 extern "C" {
 int cudaMalloc(void** p, size_t n)
 {
-    if (fake_fail_in >= 0 && fake_fail_in-- == 0) { *p = nullptr; return memory_allocation; }
+    if (fake_fail_in >= 0 && fake_fail_in-- == 0) { *p = nullptr; return last_error = memory_allocation; }
     *p = malloc(n);
     live().insert(*p);
     return ok;
@@ -23,19 +24,19 @@ int cudaMalloc(void** p, size_t n)
 int cudaFree(void* p) { live().erase(p); free(p); return ok; }
 int cudaMemcpy(void* d, const void* s, size_t n, int)
 {
-    if (!d || !s) { ++fake_null_copies; return invalid_value; }
+    if (!d || !s) { ++fake_null_copies; return last_error = invalid_value; }
     memmove(d, s, n);
     return ok;
 }
 int cudaMemcpyAsync(void* d, const void* s, size_t n, int k, void*) { return cudaMemcpy(d, s, n, k); }
 int cudaMemset(void* d, int v, size_t n)
 {
-    if (!d) { ++fake_null_copies; return invalid_value; }
+    if (!d) { ++fake_null_copies; return last_error = invalid_value; }
     memset(d, v, n);
     return ok;
 }
 int cudaMemsetAsync(void* d, int v, size_t n, void*) { return cudaMemset(d, v, n); }
-int cudaGetLastError() { return ok; }
+int cudaGetLastError() { const int e = last_error; last_error = ok; return e; }
 const char* cudaGetErrorString(int) { return "error"; }
 int cudaDeviceSynchronize() { return ok; }
 int cudaStreamSynchronize(void*) { return ok; }
