@@ -124,7 +124,8 @@ struct OneEArgs {
 };
 
 // the (m, n) and (n, m) elements of a block from the lanes that own them: element k in lane k mod 32,
-// its value in own[k / 32]
+// its value in own[k / 32].  In the block of a shell with itself both orders of a pair of functions are there, as sums
+// of the same terms in different orders: the lower triangle's gives both elements.
 template <int NA, int NB, int NOWN>
 __device__ __forceinline__ void store_block(double* __restrict__ M, const double (&own)[NOWN], const OneEArgs& s, int fa, int fb,
                                             int la0, int lb0, int n, int lane)
@@ -132,8 +133,8 @@ __device__ __forceinline__ void store_block(double* __restrict__ M, const double
 #pragma unroll
     for (int o = 0; o < NOWN; ++o) {
         const int k = lane + 32 * o;
-        if (k < NA * NB) {
-            const int i = k / NB, j = k % NB;
+        const int i = k / NB, j = k % NB;
+        if (k < NA * NB && (fa != fb || i >= j)) {
             const double v = s.fscale[fa + i] * s.fscale[fb + j] * own[o];
             M[(size_t)(la0 + i) * n + lb0 + j] = v;
             M[(size_t)(lb0 + j) * n + la0 + i] = v;
