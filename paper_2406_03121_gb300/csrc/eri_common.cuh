@@ -270,19 +270,31 @@ template <int L> __device__ __forceinline__ void boys_large_f32(float T, float* 
     }
 }
 
+// v c for a constant c that FP32 does not hold: rounded, 1/3 or sqrt(pi)/2 would move every integral to the same side, and
+// J and K sum that up.  (hi and lo are compile-time constants: one multiplication more.)
+__device__ __forceinline__ float mul_const(float v, double c)
+{
+    const float hi = (float)c, lo = (float)(c - (double)hi);
+    return fmaf(v, hi, v * lo);
+}
+
 // FP32.  The lanes of a warp lie on both sides of the grid's end, and the two sides of a branch would run one after
-// the other: the asymptote is formed for every lane (exp(-T) left out: 2e-16 at 36, below 1e-8 of 2 T F_8) and
-// replaced below the end.  For L <= 1 the lanes above it skip the rest, since the gather of rows fills the L1 data
+// the other: the asymptote is formed for every lane and replaced below the end.  It leaves out exp(-T), at most 1e-8 of 2 T F_L
+// at the end: T = 30 up to L = 5, 36 above (the asymptote, one root, carries fewer roundings than the recursion).
+// For L <= 1 the lanes above it skip the rest, since the gather of rows fills the L1 data
 // pipe there (95 % for (ss|ss)); for the longer recursions the selection is 1 to 8 % faster.  Instructions, not
 // loads, bound those, so a row holds what order 2 at a step of 1/128 needs (three FMAs, where order 4 at 1/16
 // took the upward recursion for two of its terms and a division).
 // Batch of 256 alkanes / STO-3G, per three builds: (ps|ss) 15.9 -> 12.6 ms, (ps|ps) 6.7 -> 5.8, (pp|ss) 3.3 -> 2.6,
 // (ss|ss) 10.8 -> 10.3; (H2O)_32 / 6-31G*, (ss|ss) 894 -> 733 us, (ps|ss) 1349 -> 1253.
+// Error of J and K of mixed builds against FP64, as a share of the error with the rows at 1/16 (24 geometries and densities
+// each): with the constants rounded and every end at 36, (H2O)_8 / 6-31G* 1.02 and 1.03, C7H16 / 6-31G 0.99 and 1.04;
+// as here 0.74 and 0.99, 0.93 and 1.03.  Times of the builds and the batch within 0.6 % of each other.
 template <int L> __device__ __forceinline__ void boys_f32(float T, float* F, const float4* __restrict__ tabv)
 {
-    const bool far = !(T < (float)MESS_BOYS_TMAX32);
+    const bool far = !(T < (L <= 5 ? (float)MESS_BOYS_TMAX32_L5 : (float)MESS_BOYS_TMAX32));
     const float rt = rsqrt_ftz(T), h = 0.5f * rt * rt;
-    F[0] = 0.886226925f * rt;   // sqrt(pi)/2 / sqrt(T)
+    F[0] = mul_const(rt, 0.886226925452758014);   // sqrt(pi)/2 / sqrt(T)
 #pragma unroll
     for (int m = 0; m < L; ++m) F[m + 1] = F[m] * ((float)(2 * m + 1) * h);
     if (L <= 1 && far) return;
@@ -302,7 +314,8 @@ template <int L> __device__ __forceinline__ void boys_f32(float T, float* F, con
     const float t2 = 2.0f * T;
 #pragma unroll
     for (int m = L; m >= 1; --m) {
-        d = m == 1 ? fmaf(t2, d, e) : fmaf(t2, d, e) * (1.0f / (2 * m - 1));
+        d = fmaf(t2, d, e);
+        if (m > 1) d = mul_const(d, 1.0 / (2 * m - 1));
         F[m - 1] = far ? F[m - 1] : d;
     }
 }

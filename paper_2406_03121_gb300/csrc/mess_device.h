@@ -9,6 +9,7 @@
 #define MESS_BOYS_TMAX64 48.0     // FP64: Taylor expansion below this
 #define MESS_BOYS_TMAXDF 36.0     // double-float, and the FP64 Boys function of FP32 quartets
 #define MESS_BOYS_TMAX32 36.0     // FP32
+#define MESS_BOYS_TMAX32_L5 30.0  // FP32, highest order up to 5
 #define MESS_BOYS_NF 16
 #define MESS_BOYS_NCOL (MESS_BOYS_NF + 1)
 #define MESS_BOYS_NROW 362
