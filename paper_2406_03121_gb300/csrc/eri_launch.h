@@ -59,19 +59,22 @@ inline int schwarz_lanes(int npairs)
 // Blocks over which the primitive quartets of a part's shell quartets are split (the J/K digestion is linear in
 // the integrals, so each block adds its share's): the quartets of a part on a warp (G = 32) or a block
 // (team 3) each run their primitive quartets as one chain, which a part of fewer quartets than SMs
-// leaves on a few of them.  At most two blocks per SM, and a full pass of lanes each.  Only where the whole build
+// leaves on a few of them.  At most two blocks per SM, a full pass of lanes each, and kMaxBlocks per quartet: each
+// block adds to K, so more of them round more often (one water / 6-31G, mean error of K against extended precision
+// over 48 densities: 5.9e-16 before the split and the fitted shapes, 6.4e-16 with four blocks, 7.0e-16 with up to 304; two blocks 107 us per
+// call, three or more 98).  Only where the whole build
 // has few quartets: otherwise the other parts fill the SMs, and the repeated HRR and digestion cost more
 // (kMaxBuild lies between one water / 6-31G, 1,035 quartets, 98 -> 76 us, and C2H6 / 6-31G*, 45,000, 352 -> 367).
 // One water / STO-3G in FP64: (pp|pp), one quartet of 81 primitive quartets, 80 -> 45 us, (pp|ps) 31 -> 18, the
 // whole call 115 -> 80.
 inline int prim_split(long long quartets, long long prim_quartets, int G, int team, long long build_quartets)
 {
-    constexpr long long kMaxBuild = 16384;
+    constexpr long long kMaxBuild = 16384, kMaxBlocks = 4;
     if (build_quartets > kMaxBuild) return 1;
     const int lanes = team == 3 ? MESS_TEAM_WARPS : (G == 32 && !team ? 32 : 0);
     if (!lanes || quartets <= 0 || quartets > 152) return 1;
     const long long passes = (prim_quartets / quartets + lanes - 1) / lanes;
-    return (int)std::max(1LL, std::min(passes, 2 * 152 / quartets));
+    return (int)std::max(1LL, std::min({passes, 2 * 152 / quartets, kMaxBlocks}));
 }
 
 typedef cudaError_t (*mess_class_launcher)(const ClassLaunchArgs&);
