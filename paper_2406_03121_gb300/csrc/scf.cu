@@ -337,11 +337,9 @@ __device__ __forceinline__ float jac_f32(df32 x) { return x.hi; }
 template <typename T> __device__ __forceinline__ T jac_const(float v);
 template <> __device__ __forceinline__ double jac_const<double>(float v) { return v; }
 template <> __device__ __forceinline__ df32 jac_const<df32>(float v) { return df32(v, 0.f); }
-// sums of squares for the convergence test: FP64, or FP32 where the threshold is only 1e-25 of the whole
-template <typename T> struct JacSum { typedef double type; };
-template <> struct JacSum<df32> { typedef float type; };
+// square for the convergence test, summed in FP64 (once per sweep, beside its n rounds)
 __device__ __forceinline__ double jac_sq(double x) { return x * x; }
-__device__ __forceinline__ float jac_sq(df32 x) { return x.hi * x.hi; }
+__device__ __forceinline__ double jac_sq(df32 x) { return jac_sq(f2d_alu(x.hi)); }
 // cosine of the rotation whose tangent is t: (1 + t^2)^(-1/2) to the element type's accuracy
 __device__ __forceinline__ double jac_cos(double, float t) { return rsqrt(fma((double)t, (double)t, 1.0)); }
 __device__ __forceinline__ df32 jac_cos(df32, float t)
@@ -404,7 +402,6 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
     __shared__ unsigned char pp2[2][kJacMaxHalf], qq2[2][kJacMaxHalf], on2[2][kJacMaxHalf];   // (round parity)
     __shared__ __align__(16) unsigned char cc_raw[2 * kJacMaxHalf * sizeof(T)], ss_raw[2 * kJacMaxHalf * sizeof(T)];
     __shared__ int rotated;
-    typedef typename JacSum<T>::type Sum;
     const int m = blockIdx.x;
     if (!L.active[m]) return;
     const int n = L.n[m];
@@ -461,7 +458,7 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
             on2[par][k] = (unsigned char)(q < n ? on : 2);      // 2: the pair of the padding index
         }
     };
-    Sum nrm = 0;
+    double nrm = 0.0;
     for (int i = warp; i < n; i += nwarp)
         for (int j = lane; j < n; j += 32) {
             Vt[i * n + j] = (i == j) ? one : zero;
@@ -471,13 +468,13 @@ __global__ void __launch_bounds__(512) k_jacobi(const double* __restrict__ Ain, 
             A[i * pitch + j] = v;
             nrm += i == j ? jac_sq(v) : 2 * jac_sq(v);
         }
-    const double norm2 = block_sum((double)nrm, red);   // (synchronises the block)
+    const double norm2 = block_sum(nrm, red);   // (synchronises the block)
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
-        Sum off = 0;
+        double off = 0.0;
         for (int i = warp; i < n; i += nwarp)
             for (int j = i + 1 + lane; j < n; j += 32) off += 2 * jac_sq(A[i * pitch + j]);
-        const double off2 = block_sum((double)off, red);
+        const double off2 = block_sum(off, red);
         if (off2 <= JacEps<T>::off * norm2 || off2 == 0.0) break;
         if (threadIdx.x == 0) rotated = 0;
         __syncthreads();
