@@ -34,7 +34,7 @@ void mess_boys_table(std::vector<double>& tab, int nrow, double dt)
 }
 
 // The kernels' tables (mess_device.h): constants, the same for every basis, so one copy per device in the
-// library's image, filled when the first basis of the device builds its data (2.0 MB; tabulating them
+// library's image, filled when the first basis of the device builds its data (2.5 MB; tabulating them
 // for every basis took 6 ms of host time each).
 static __device__ __align__(256) double g_boys64[MESS_BOYS_NL * MESS_BOYS64_NROW * 8];
 static __device__ __align__(256) float4 g_boys32[MESS_BOYS_NL * MESS_BOYS32_NROW];

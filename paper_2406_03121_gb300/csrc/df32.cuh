@@ -62,28 +62,11 @@ __device__ __forceinline__ df32u operator*(df32 a, df32 b)
     return df32u(p, e);
 }
 
-__device__ __forceinline__ df32 operator/(df32 a, df32 b)
-{
-    const float q1 = __fdividef(a.hi, b.hi);
-    const df32 r = a - b * df32(q1, 0.f);
-    const float q2 = __fdividef(r.hi, b.hi);
-    return df_fast_two_sum(q1, q2);
-}
-
 __device__ __forceinline__ df32& operator+=(df32& a, df32u b) { a = a + b; return a; }
 __device__ __forceinline__ df32& operator-=(df32& a, df32u b) { a = a - b; return a; }
 __device__ __forceinline__ df32& operator*=(df32& a, df32 b) { a = a * b; return a; }
 __device__ __forceinline__ bool operator!=(df32 a, df32 b) { return a.hi != b.hi || a.lo != b.lo; }
 __device__ __forceinline__ bool operator<(df32 a, double b) { return a.hi < (float)b; }
-
-// sqrt by one Newton correction of the FP32 root: s + (a - s^2) / (2 s)
-__device__ __forceinline__ df32 df_sqrt(df32 a)
-{
-    if (a.hi <= 0.f) return df32(0.f, 0.f);
-    const float s = sqrtf(a.hi);
-    const df32 r = a - df32(s, 0.f) * df32(s, 0.f);
-    return df_fast_two_sum(s, __fdividef(r.hi, 2.f * s));
-}
 
 // a + b for |a| >= |b| (8 instructions instead of 11)
 __device__ __forceinline__ df32 df_add_smaller(df32 a, df32u b)

@@ -11,12 +11,15 @@
 // digestion, fix = h + g, and where G lanes deal out the digestion h + g / G (G = 1 for the team kernels).
 // The constants (microseconds) are fitted by least squares on the logarithm to 4000 such timings on one
 // GB300: every class and shape, 1 to 13 million quartets, 1 to 420 primitive quartets each, from one water
-// in STO-3G to (H2O)_32 in 6-31G*; one timing is estimated within 12 to 33 % (one standard deviation).
-// Summed over the parts of a build, the chosen shapes take 541, 5669, 2293, 3019 and 27880 us for C2H6 and
-// (H2O)_8 (FP64), (H2O)_8, C7H16 and (H2O)_32 (mixed), where the best shape of every part, found by timing
-// them all, takes 527, 5515, 2204, 2882 and 27223 us.  Against the fixed thresholds on quartets and
-// primitives that stood here before, whole builds: one water 251 -> 115 us, (H2O)_8 6.8 -> 4.8 ms (FP64), (H2O)_8
-// 1.48 -> 1.03, C7H16 1.19 -> 0.94 and (H2O)_32 16.3 -> 16.0 ms (mixed).
+// in STO-3G to (H2O)_32 in 6-31G*; one timing was estimated within 12 to 33 % (one standard deviation).
+// The timings are of the kernels before the bra runs (MESS_RUN_MIN), the finer FP32 Boys rows, the double-float sums
+// normalised once per expression (8 to 23 % faster) and the split of primitive quartets over blocks (prim_split). The
+// estimate has no terms for runs and that split: a part in runs (up to 3.3 times faster) is ordered and put on a stream by
+// the time of one thread per quartet. With the kernels of the fit, summed over the parts of a build,
+// the chosen shapes took 541, 5669, 2293, 3019 and 27880 us for C2H6 and (H2O)_8 (FP64), (H2O)_8, C7H16 and (H2O)_32
+// (mixed), where the best shape of every part, found by timing them all, took 527, 5515, 2204, 2882 and 27223 us.
+// Against fixed thresholds on quartets and primitives, whole builds: one water 251 -> 115 us, (H2O)_8 6.8 -> 4.8 ms
+// (FP64), (H2O)_8 1.48 -> 1.03, C7H16 1.19 -> 0.94 and (H2O)_32 16.3 -> 16.0 ms (mixed).
 #pragma once
 #include <math.h>
 

@@ -140,7 +140,7 @@ struct JKGraph {
 struct XcState {
     bool ready = false;
     long long npts = 0, ao = 0, mol_npts_max = 0;
-    DevBuf<double> pts, w, phi, dphi, vrho, vgrad, Exc, tab;
+    DevBuf<double> pts, w, phi, dphi, vrho, vgrad, tab;
     DevBuf<int> atom, atom_mol, radial_at, radial_n, fbase, shell_off, shell_n, shell_fl;
     DevBuf<long long> pbase, aobase, abase;
 };

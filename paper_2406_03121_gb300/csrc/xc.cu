@@ -206,8 +206,10 @@ __global__ void k_ao(AoArgs a)
 }
 
 // Roots, reciprocals and logarithms of the functional in few FP64 instructions (each takes 16 cycles of an
-// SM; the library's log1p, rcbrt, sqrt and division took most of an LDA point's): an FP32
-// estimate, relative error e below 1e-5, and the first terms of the series in e, whose next is below 1e-17.
+// SM; the library's log1p, rcbrt, sqrt and division took most of an LDA point's): an FP32 estimate and the first
+// terms of the series in what it leaves, e.  Reciprocal and reciprocal root: e below 4e-7 (the roundings to FP32 and
+// the estimate's), and the next term, in e^3, below 1e-19.  Cube root, by exp2 of a third of log2 x, which is rounded in
+// proportion to its size (up to 100): e below 1e-5 at the ends of the range and 3e-6 about x = 1, next term 2e-16 and 1e-17.
 // x^(-1/3) for 1e-14 <= x (an FP32 number): (1 - e)^(-1/3) = 1 + e/3 + 2/9 e^2, e = 1 - x y^3
 __device__ __forceinline__ double inv_cbrt(double x)
 {
@@ -608,7 +610,7 @@ void mess_free_xc(mess_basis* b)
     x.pts.free(); x.w.free(); x.atom.free(); x.atom_mol.free(); x.tab.free(); x.radial_at.free(); x.radial_n.free();
     x.abase.free(); x.pbase.free(); x.phi.free(); x.dphi.free();
     x.aobase.free(); x.vrho.free(); x.vgrad.free(); x.fbase.free(); x.shell_off.free(); x.shell_n.free();
-    x.shell_fl.free(); x.Exc.free();
+    x.shell_fl.free();
     x.npts = 0;
     x.ready = false;
 }
@@ -694,7 +696,6 @@ mess_status mess_xc_prepare(mess_basis* b, cudaStream_t s)
     MESS_CUDA_TRY(X.dphi.alloc((size_t)ao * 3));
     MESS_CUDA_TRY(X.vrho.alloc((size_t)X.npts));
     MESS_CUDA_TRY(X.vgrad.alloc((size_t)X.npts * 3));
-    MESS_CUDA_TRY(X.Exc.alloc((size_t)b->nmol));
     const int T = 256;
     const unsigned blocks = (unsigned)((X.npts + T - 1) / T);
     k_grid<<<(unsigned)(b->natom * kBlocksPerAtom), kGridThreads, 0, s>>>(X.tab.p, X.radial_at.p, X.radial_n.p, X.abase.p,
