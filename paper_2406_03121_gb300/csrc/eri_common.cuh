@@ -289,7 +289,8 @@ __device__ __forceinline__ float mul_const(float v, double c)
 // (ss|ss) 10.8 -> 10.3; (H2O)_32 / 6-31G*, (ss|ss) 894 -> 733 us, (ps|ss) 1349 -> 1253.
 // Error of J and K of mixed builds against FP64, as a share of the error with the rows at 1/16 (24 geometries and densities
 // each): with the constants rounded and every end at 36, (H2O)_8 / 6-31G* 1.02 and 1.03, C7H16 / 6-31G 0.99 and 1.04;
-// as here 0.74 and 0.99, 0.93 and 1.03.  Times of the builds and the batch within 0.6 % of each other.
+// as here 0.74 and 0.99, 0.93 and 1.03 (0.74 and 0.96, 0.93 and 0.95 with the lanes' sums rounded once, lane_sum).
+// Times of the builds and the batch within 0.6 % of each other.
 template <int L> __device__ __forceinline__ void boys_f32(float T, float* F, const float4* __restrict__ tabv)
 {
     const bool far = !(T < (L <= 5 ? (float)MESS_BOYS_TMAX32_L5 : (float)MESS_BOYS_TMAX32));
@@ -438,29 +439,41 @@ __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sy
 __device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ df32 shfl_xor(df32 v, int o) { return df_shfl_xor(v, o); }
 
+// a + b of two lanes, and the rounding of a whole sum.  FP32 values are summed as hi + lo and rounded once: log2 G roundings
+// at the size of the sum move K more than a lane's whole chain of primitives does.  Error of K of C7H16 / 6-31G below
+// the split, all classes with 32 lanes, 2.85e-10 -> 2.44e-10 (8 lanes 2.85 -> 2.51, 4 lanes 2.78 -> 2.52, one thread 2.57);
+// mixed builds take 0 to 0.7 % longer.
+__device__ __forceinline__ df32 lane_sum(float a, float b) { return df_two_sum(a, b); }
+__device__ __forceinline__ df32 lane_sum(df32 a, df32 b) { return a + b; }
+__device__ __forceinline__ double lane_sum(double a, double b) { return a + b; }
+__device__ __forceinline__ void lane_store(float& x, float v) { x = v; }
+__device__ __forceinline__ void lane_store(float& x, df32 v) { x = v.hi + v.lo; }
+__device__ __forceinline__ void lane_store(df32& x, df32 v) { x = v; }
+__device__ __forceinline__ void lane_store(double& x, double v) { x = v; }
+
 // Sums of acc[0..N) over the G lanes of a group into the group's shared array sh.  Each halving of the
 // group also halves what a lane carries on (it keeps one half and sends the other), so the whole costs
 // about N additions per lane; an all-lanes butterfly of every value takes N log2 G.
 template <int O, int N> struct GroupSums {
-    template <typename R> static __device__ __forceinline__ void run(const R (&acc)[N], int g, int off, int len, R* sh)
+    template <typename R, typename S> static __device__ __forceinline__ void run(const R (&acc)[N], int g, int off, int len, S* sh)
     {
         constexpr int H = (N + 1) / 2;
         const bool up = (g & O) != 0;
-        R t[H];
+        decltype(lane_sum(acc[0], acc[0])) t[H];
 #pragma unroll
         for (int k = 0; k < H; ++k) {
             const R lo = acc[k], hi = k + H < N ? acc[k + H < N ? k + H : 0] : R(0);
-            t[k] = (up ? hi : lo) + shfl_xor(up ? lo : hi, O);
+            t[k] = lane_sum(up ? hi : lo, shfl_xor(up ? lo : hi, O));
         }
         GroupSums<O / 2, H>::run(t, g, up ? off + H : off, up ? max(len - H, 0) : min(len, H), sh);
     }
 };
 template <int N> struct GroupSums<0, N> {
-    template <typename R> static __device__ __forceinline__ void run(const R (&acc)[N], int, int off, int len, R* sh)
+    template <typename R, typename S> static __device__ __forceinline__ void run(const R (&acc)[N], int, int off, int len, S* sh)
     {
 #pragma unroll
         for (int k = 0; k < N; ++k)
-            if (k < len) sh[off + k] = acc[k];
+            if (k < len) lane_store(sh[off + k], acc[k]);
     }
 };
 
